@@ -23,7 +23,8 @@
 // The propagator multiply sits in pass C; the inverse runs the passes back
 // (C, B, A) with conjugate twiddles, so no index permutation is ever stored.
 // Between passes the data crosses threads through one shared table in which
-// every thread writes only the entries it has just read (four barriers per
+// every thread writes only the entries it has just read. A warp owns the same rows
+// in passes A and B, so only the exchanges with pass C need CTA barriers (two per
 // slice); each warp stages the transmission rows it multiplies into its own
 // table rows with cp.async while its inverse pass A runs. The transmission is
 // stored with a periodic halo of W pixels ([ny + W][nx + W] per slice), so
@@ -431,24 +432,31 @@ __device__ __forceinline__ void load_twiddles(float2* twA, float2* twB, int T) {
 // ------------------------------------------------------------------------------------------
 // step a3: slice kernel
 // ------------------------------------------------------------------------------------------
-// The slice kernel keeps every exchange in one table of 512 rows x 34 entries (row TA =
-// 4 y + r, entry k), and every thread writes only the entries it has just read:
+// The slice kernel keeps every exchange in one table of 512 rows x 34 entries (row TA = 16 n2y
+// + 4 n1y + r for window row y = 32 n1y + n2y, entry k), and every thread writes only the
+// entries it has just read:
 //   A thread (y, r):   row TA = T, entries 0..31: its pass-A outputs k1 (X1), later its
 //                      pass-B-inverse inputs (X4)
-//   B thread (k1, n2y): entries k1 of rows 4 (32 q + n2y) + r, q, r < 4: X1 element
-//                      (y = 32 q + n2y, r, k1) at slot (q, r); its pass-B output (k1y, k2x)
-//                      goes to slot (q, r) = (k2x, k1y) (X2) and its inverse output
-//                      (q, r) back to slot (q, r) (X4)
-//   C thread (kx, k1y): entry k1x of rows 4 (32 k2x + j) + k1y, j < 32 (read, write back)
-//   warp w:            rows 32 w .. 32 w + 31 (1056 entries) also hold the transmission
-//                      of its 8 window rows y = 8 w .. 8 w + 7 as 8 rows of 132 entries
-// No entry is written by one thread while another thread of the CTA may still read it,
-// so the only CTA barriers are the four that publish a phase's writes (read-after-write);
-// the transmission is shared within a warp only (__syncwarp). With rows of 34 entries the
-// A side moves entry pairs (k, k + 1) with 128-bit accesses, a quarter-warp's 8 rows on 8
-// distinct 16-byte slots (17 TA + k/2 mod 8); the 64-bit B and C accesses of a half-warp
-// are 16 consecutive entries of one row (of two rows 128 x 34 entries apart in the warps
-// that mix k2x), on 16 distinct bank pairs.
+//   B thread (k1, n2y): entries k1 of rows 16 n2y + 4 q + r, q, r < 4: X1 element (y = 32 q +
+//                      n2y, r, k1) at slot (q, r); its pass-B output (k1y, k2x) goes to slot
+//                      (q, r) = (x2_slot(k2x), k1y) (X2) and its inverse output (q, r) back to
+//                      slot (q, r) (X4)
+//   C thread (kx, k1y): entry k1x of rows 16 j + 4 x2_slot(k2x) + k1y, j < 32 (read, write back)
+//   warp w:            rows 32 w .. 32 w + 31 (1088 entries) also hold the transmission of
+//                      its 8 window rows y = 32 q + 2 w + h (q < 4, h < 2) as 8 rows of 132 entries
+// A warp's 8 window rows are the 4 n1y of two n2y, so pass A and pass B of one warp read and
+// write the same 32 table rows: X1, X4 and the transmission need only __syncwarp, and the CTA
+// barriers are the two that publish X2 to pass C and X3 back. Between them a warp runs inverse
+// B and A, the transmission and forward A and B at its own pace, so that the exchanges of some
+// warps overlap the arithmetic of others. With warps of 8 consecutive window rows, X1 and X4
+// crossed warps (four barriers a slice) and the phases of all 16 warps ran in step: 320 ms
+// per 131072 translates x 50 slices, 291 ms since.
+// With rows of 34 entries the A side moves entry pairs (k, k + 1) with 128-bit accesses, a
+// quarter-warp's 8 rows on 8 distinct 16-byte slots (17 TA + k/2 mod 8); the 64-bit B and C
+// accesses of a half-warp are 16 consecutive entries of one row, on 16 distinct bank pairs (of
+// two rows 8 apart in the warps that mix k2x = 1 and 2: 8 x 34 entries are a multiple of 16,
+// which is why x2_slot exchanges k2x = 2 and 3).
+__host__ __device__ constexpr int x2_slot(int k2x) { return k2x < 2 ? k2x : 5 - k2x; }
 constexpr int kXP = 34;
 constexpr int kXRows = 512 * kXP;
 constexpr int kTRow = 132;   // staged transmission row: 4 table rows
@@ -460,9 +468,9 @@ constexpr int kPRow = 65;
 constexpr int kPTab = kPRow * kPRow;
 constexpr int kSliceSmemFloat2 = kXRows + 128 + 128 + kPTab;
 
-// Warp w copies window rows 8 w .. 8 w + 7 of one slice (g points at the first) into its
-// table rows (asynchronous; the warp's threads read them after cp_async_wait_all and
-// __syncwarp). With an even window origin in 16-byte pieces, 512 contiguous bytes per
+// Warp w copies its window rows y = 32 (i & 3) + 2 w + (i >> 2), i < 8, of one slice (g points
+// at row 2 w) into its table rows (asynchronous; the warp's threads read them after
+// cp_async_wait_all and __syncwarp). With an even window origin in 16-byte pieces, 512 contiguous bytes per
 // instruction; with an odd origin in 8-byte pieces.
 template <bool EVEN>
 __device__ __forceinline__ void stage_t_warp(float2* region, const float2* g, int pitch, int lane) {
@@ -470,13 +478,13 @@ __device__ __forceinline__ void stage_t_warp(float2* region, const float2* g, in
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
       const int yl = i >> 1, x = 64 * (i & 1) + 2 * lane;
-      cp_async16(region + yl * kTRow + x, g + static_cast<size_t>(yl) * pitch + x);
+      cp_async16(region + yl * kTRow + x, g + static_cast<size_t>(32 * (yl & 3) + (yl >> 2)) * pitch + x);
     }
   } else {
 #pragma unroll
     for (int i = 0; i < 32; ++i) {
       const int yl = i >> 2, x = 32 * (i & 3) + lane;
-      cp_async8(region + yl * kTRow + x, g + static_cast<size_t>(yl) * pitch + x);
+      cp_async8(region + yl * kTRow + x, g + static_cast<size_t>(32 * (yl & 3) + (yl >> 2)) * pitch + x);
     }
   }
   cp_async_commit();
@@ -498,8 +506,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_slice(const SliceLaunch a, cons
   const int T = threadIdx.x;
   if (T < 128) twB[T] = c_w128[((T >> 2) * (T & 3)) & 127];
   if (T < 64) twr[T] = T < 32 ? c_twrA[T] : c_twrB[T - 32];
-  // A layout: thread (y, r), TA = T
-  const int ya = T >> 2, ra = T & 3;
+  // A layout: thread (y, r), y = 32 n1y + n2y, T = 16 n2y + 4 n1y + r
+  const int ya = 32 * ((T >> 2) & 3) + (T >> 4), ra = T & 3;
   // B layout: groups (k1 = (T & 15) + 16 h, n2y = T >> 4), h = 0, 1
   const int k1lo = T & 15, n2y = T >> 4;
   // C layout: thread (kx, k1y), kx permuted within each k1y group (c_column)
@@ -514,11 +522,11 @@ __global__ void __launch_bounds__(kThreads, 1) k_slice(const SliceLaunch a, cons
   __shared__ int s_next;
   __shared__ int s_wmax;      // FP16 store: bits of the wave's largest |component| (order-preserving for >= 0)
   float2* const xa = X + T * kXP;                                 // A row, + n or k1
-  float2* const xb = X + (4 * n2y) * kXP + k1lo;                  // B slot (q, r): + (128 q + r) * kXP, + 16 (h = 1)
-  float2* const xc = X + (128 * k2x + k1y) * kXP + k1x;           // C entry j: + 4 j * kXP
+  float2* const xb = X + (16 * n2y) * kXP + k1lo;                 // B slot (q, r): + (4 q + r) * kXP, + 16 (h = 1)
+  float2* const xc = X + (4 * x2_slot(k2x) + k1y) * kXP + k1x;    // C entry j: + 16 j * kXP
   const int lane = T & 31;
   float2* const xw = X + (T >> 5) * (32 * kXP);                   // this warp's table rows
-  const float2* const tr = xw + (ya & 7) * kTRow + ra;            // t(y, 4 n + r) at + 4 n
+  const float2* const tr = xw + (lane >> 2) * kTRow + ra;         // t(y, 4 n + r) at + 4 n
 
   __syncthreads();   // twiddles
 
@@ -537,7 +545,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_slice(const SliceLaunch a, cons
     while (jb + 1 < a.n_jobs && li >= a.start[jb + 1]) ++jb;
     const SliceJob& J = a.job[jb];
     if (jb != cur_job) {
-      // the previous item's last barrier has passed: the table is free; the X1 barrier
+      // the previous item's last barrier has passed: the table is free; the X2 barrier
       // below publishes it before pass C reads it
       cur_job = jb;
       for (int e = T; e < kPTab; e += kThreads) {
@@ -559,7 +567,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_slice(const SliceLaunch a, cons
     int oy = (J.lat_oy + ib * J.lat_sy - kW / 2) % J.ny;
     if (oy < 0) oy += J.ny;
     // the halo of W pixels keeps every window inside the padded array
-    const float2* const gsrc = J.t + cfg * J.t_slot + static_cast<size_t>(oy + 8 * (T >> 5)) * pitch + ox;
+    const float2* const gsrc = J.t + cfg * J.t_slot + static_cast<size_t>(oy + 2 * (T >> 5)) * pitch + ox;
 
     stage_t_warp<EVEN>(xw, gsrc, pitch, lane);
     float2 v[32];
@@ -579,32 +587,32 @@ __global__ void __launch_bounds__(kThreads, 1) k_slice(const SliceLaunch a, cons
       float4* const xa4 = reinterpret_cast<float4*>(xa);
 #pragma unroll
       for (int k = 0; k < 32; k += 2) xa4[k / 2] = make_float4(v[k].x, v[k].y, v[k + 1].x, v[k + 1].y);
-      __syncthreads();
+      __syncwarp();
       float2 b0[16], b1[16];
 #pragma unroll
       for (int q = 0; q < 4; ++q)
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-          b0[q * 4 + r] = xb[(128 * q + r) * kXP];
-          b1[q * 4 + r] = xb[(128 * q + r) * kXP + 16];
+          b0[q * 4 + r] = xb[(4 * q + r) * kXP];
+          b1[q * 4 + r] = xb[(4 * q + r) * kXP + 16];
         }
       passB_fwd_tw<false, PRUNE>(b0, tB, twr[k1lo], twr[32 + k1lo]);
       passB_fwd_tw<true, PRUNE>(b1, tB, twr[16 + k1lo], twr[48 + k1lo]);
-      // X2: element (k1y, k2x) to slot (q, r) = (k2x, k1y); a pruned column is not written
+      // X2: element (k1y, k2x) to slot (x2_slot(k2x), k1y); a pruned column is not written
       // (pass C finds finite values of this slice's X1 there and multiplies them by zero)
       static_for<0, 4>([&](auto qq) {
         constexpr int q = decltype(qq)::value;
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-          if constexpr (q != masked_k2x<false, PRUNE>()) xb[(128 * q + r) * kXP] = b0[r * 4 + q];
-          if constexpr (q != masked_k2x<true, PRUNE>()) xb[(128 * q + r) * kXP + 16] = b1[r * 4 + q];
+          if constexpr (q != masked_k2x<false, PRUNE>()) xb[(4 * x2_slot(q) + r) * kXP] = b0[r * 4 + q];
+          if constexpr (q != masked_k2x<true, PRUNE>()) xb[(4 * x2_slot(q) + r) * kXP + 16] = b1[r * 4 + q];
         }
       });
       __syncthreads();
       if (c_live) {
         float2 c[32];
 #pragma unroll
-        for (int j = 0; j < 32; ++j) c[j] = xc[j * 4 * kXP];
+        for (int j = 0; j < 32; ++j) c[j] = xc[j * 16 * kXP];
         dft32<false, PRUNE ? 1 : 0>(c);
         // propagation (Sec. 3.2): exp(-i pi lambda eps |k|^2), bandlimit, 1/W^2
 #pragma unroll
@@ -612,18 +620,19 @@ __global__ void __launch_bounds__(kThreads, 1) k_slice(const SliceLaunch a, cons
           if (!PRUNE || !in_gap(j)) c[j] = cmul(c[j], j < 16 ? pp[4 * j] : pm[-4 * j]);
         dft32<true, PRUNE ? 2 : 0>(c);
 #pragma unroll
-        for (int j = 0; j < 32; ++j) xc[j * 4 * kXP] = c[j];
-      } else {
+        for (int j = 0; j < 32; ++j) xc[j * 16 * kXP] = c[j];
+      } else if (!PRUNE || (k2x == 1 && k1x < 16)) {
+        // with PRUNE, pass B reads no other masked column of these warps (masked_k2x)
 #pragma unroll
-        for (int j = 0; j < 32; ++j) xc[j * 4 * kXP] = make_float2(0.f, 0.f);
+        for (int j = 0; j < 32; ++j) xc[j * 16 * kXP] = make_float2(0.f, 0.f);
       }
       __syncthreads();
       static_for<0, 4>([&](auto qq) {
         constexpr int q = decltype(qq)::value;
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-          if constexpr (q != masked_k2x<false, PRUNE>()) b0[r * 4 + q] = xb[(128 * q + r) * kXP];
-          if constexpr (q != masked_k2x<true, PRUNE>()) b1[r * 4 + q] = xb[(128 * q + r) * kXP + 16];
+          if constexpr (q != masked_k2x<false, PRUNE>()) b0[r * 4 + q] = xb[(4 * x2_slot(q) + r) * kXP];
+          if constexpr (q != masked_k2x<true, PRUNE>()) b1[r * 4 + q] = xb[(4 * x2_slot(q) + r) * kXP + 16];
         }
       });
       passB_inv_tw<false, PRUNE>(b0, tB, twr[k1lo], twr[32 + k1lo]);
@@ -633,10 +642,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_slice(const SliceLaunch a, cons
       for (int q = 0; q < 4; ++q)
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-          xb[(128 * q + r) * kXP] = b0[q * 4 + r];
-          xb[(128 * q + r) * kXP + 16] = b1[q * 4 + r];
+          xb[(4 * q + r) * kXP] = b0[q * 4 + r];
+          xb[(4 * q + r) * kXP + 16] = b1[q * 4 + r];
         }
-      __syncthreads();
+      __syncwarp();
       {
         const float4* const xa4 = reinterpret_cast<const float4*>(xa);
 #pragma unroll
@@ -674,13 +683,13 @@ __global__ void __launch_bounds__(kThreads, 1) k_slice(const SliceLaunch a, cons
       // 16 bytes apart in the wave, so direct stores would write half sectors)
       __half2* const hs = reinterpret_cast<__half2*>(xw);
 #pragma unroll
-      for (int n1 = 0; n1 < 32; ++n1) hs[(ya & 7) * 132 + 4 * n1 + ra] = __floats2half2_rn(v[n1].x * sc, v[n1].y * sc);
+      for (int n1 = 0; n1 < 32; ++n1) hs[(lane >> 2) * 132 + 4 * n1 + ra] = __floats2half2_rn(v[n1].x * sc, v[n1].y * sc);
       __syncwarp();
       uint4* const dst = reinterpret_cast<uint4*>(static_cast<__half2*>(J.Uh) + cfg * J.u_slot +
-                                                  static_cast<size_t>(oi) * (kW * kW) + (8 * (T >> 5)) * kW);
+                                                  static_cast<size_t>(oi) * (kW * kW) + (2 * (T >> 5)) * kW);
 #pragma unroll
       for (int yl = 0; yl < 8; ++yl)
-        dst[yl * (kW / 4) + lane] = *reinterpret_cast<const uint4*>(hs + yl * 132 + 4 * lane);
+        dst[(32 * (yl & 3) + (yl >> 2)) * (kW / 4) + lane] = *reinterpret_cast<const uint4*>(hs + yl * 132 + 4 * lane);
       if (T == 0) J.Uscale[static_cast<size_t>(cfg) * J.n_translates + oi] = ldexpf(1.f, e);
     } else {
       const int oi = a.out_index ? a.out_index[li] : ti;
@@ -890,10 +899,10 @@ constexpr int kSliceTcSmemBytes = kXRows * 8 + 4 * tc::kBBytes + 64 * 16 + 128 *
 // accumulator is TMEM columns 64 t .. 64 t + 63. Each tile synchronizes its 128 threads with
 // a named barrier, one elected thread issues the tile's MMAs and commits them to the tile's
 // mbarrier, and the tile's threads read their rows back as soon as it completes: the tensor
-// cores work on one tile while the CUDA cores split, store or read back the others. CTA
-// barriers remain where data cross tiles: the pass-B exchanges (X1..X4), the reads of X2
-// before pass C's operands overwrite the table, and the X3 writes after every tile's
-// inverse pass C.
+// cores work on one tile while the CUDA cores split, store or read back the others. A warp's
+// rows are the same in passes A and B (as in k_slice: X1 and X4 need __syncwarp). CTA
+// barriers remain where data cross tiles: X2 and X3, the reads of X2 before pass C's operands
+// overwrite the table, and the X3 writes after every tile's inverse pass C.
 template <bool EVEN, bool PRUNE>
 __global__ void __launch_bounds__(kThreads, 1) k_slice_tc(const SliceLaunch a, int* status) {
   extern __shared__ __align__(1024) unsigned char smraw[];
@@ -933,7 +942,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_slice_tc(const SliceLaunch a, i
   unsigned char* const aLo = aHi + tc::kHalfBytes;
   const int arow = T & 127;
 
-  const int ya = T >> 2, ra = T & 3;
+  const int ya = 32 * ((T >> 2) & 3) + (T >> 4), ra = T & 3;   // rows and exchange slots as in k_slice
   const int k1lo = T & 15, n2y = T >> 4;
   const int kx = c_column(T), k1y = T >> 7, k1x = kx & 31, k2x = kx >> 5;
   const float2* tB = twB + n2y * 4;
@@ -943,10 +952,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_slice_tc(const SliceLaunch a, i
   bool c_live = false;
   int cur_job = -1;
   float2* const xa = X + T * kXP;
-  float2* const xb = X + (4 * n2y) * kXP + k1lo;
-  float2* const xc = X + (128 * k2x + k1y) * kXP + k1x;
+  float2* const xb = X + (16 * n2y) * kXP + k1lo;
+  float2* const xc = X + (4 * x2_slot(k2x) + k1y) * kXP + k1x;
   float2* const xw = X + (T >> 5) * (32 * kXP);
-  const float2* const tr = xw + (ya & 7) * kTRow + ra;
+  const float2* const tr = xw + (lane >> 2) * kTRow + ra;
   uint32_t phase = 0;   // parity of the next round of every tile's mbarrier
   // a wait that gives up sets `bad`; the TMEM load after it still reads this CTA's own
   // columns (values of no use), and the next CTA barrier (__syncthreads_or) abandons the launch
@@ -995,7 +1004,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_slice_tc(const SliceLaunch a, i
     if (ox < 0) ox += J.nx;
     int oy = (J.lat_oy + ib * J.lat_sy - kW / 2) % J.ny;
     if (oy < 0) oy += J.ny;
-    const float2* const gsrc = J.t + cfg * J.t_slot + static_cast<size_t>(oy + 8 * (T >> 5)) * pitch + ox;
+    const float2* const gsrc = J.t + cfg * J.t_slot + static_cast<size_t>(oy + 2 * (T >> 5)) * pitch + ox;
 
     stage_t_warp<EVEN>(xw, gsrc, pitch, lane);
     float2 v[32];
@@ -1024,14 +1033,14 @@ __global__ void __launch_bounds__(kThreads, 1) k_slice_tc(const SliceLaunch a, i
       float4* const xa4 = reinterpret_cast<float4*>(xa);
 #pragma unroll
       for (int k = 0; k < 32; k += 2) xa4[k / 2] = make_float4(v[k].x, v[k].y, v[k + 1].x, v[k + 1].y);
-      if (__syncthreads_or(bad)) goto abort;
+      __syncwarp();
       float2 b0[16], b1[16];
 #pragma unroll
       for (int q = 0; q < 4; ++q)
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-          b0[q * 4 + r] = xb[(128 * q + r) * kXP];
-          b1[q * 4 + r] = xb[(128 * q + r) * kXP + 16];
+          b0[q * 4 + r] = xb[(4 * q + r) * kXP];
+          b1[q * 4 + r] = xb[(4 * q + r) * kXP + 16];
         }
       passB_fwd_tw<false, PRUNE>(b0, tB, twr[k1lo], twr[32 + k1lo]);
       passB_fwd_tw<true, PRUNE>(b1, tB, twr[16 + k1lo], twr[48 + k1lo]);
@@ -1039,16 +1048,16 @@ __global__ void __launch_bounds__(kThreads, 1) k_slice_tc(const SliceLaunch a, i
         constexpr int q = decltype(qq)::value;
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-          if constexpr (q != masked_k2x<false, PRUNE>()) xb[(128 * q + r) * kXP] = b0[r * 4 + q];
-          if constexpr (q != masked_k2x<true, PRUNE>()) xb[(128 * q + r) * kXP + 16] = b1[r * 4 + q];
+          if constexpr (q != masked_k2x<false, PRUNE>()) xb[(4 * x2_slot(q) + r) * kXP] = b0[r * 4 + q];
+          if constexpr (q != masked_k2x<true, PRUNE>()) xb[(4 * x2_slot(q) + r) * kXP + 16] = b1[r * 4 + q];
         }
       });
-      __syncthreads();
+      if (__syncthreads_or(bad)) goto abort;
       // pass C forward: every row of X2 is read before the operands overwrite the table
       float2 c[32];
       if (c_live) {
 #pragma unroll
-        for (int j = 0; j < 32; ++j) c[j] = xc[j * 4 * kXP];
+        for (int j = 0; j < 32; ++j) c[j] = xc[j * 16 * kXP];
       }
       __syncthreads();
       if (c_live) tc::store_row(aHi, aLo, c, arow);
@@ -1068,10 +1077,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_slice_tc(const SliceLaunch a, i
         if (u != tile) bad |= !tc::wait_phase_warp(tc::smem_u32(mbar + u), phase ^ 1);
       if (c_live) {
 #pragma unroll
-        for (int j = 0; j < 32; ++j) xc[j * 4 * kXP] = c[j];
-      } else {
+        for (int j = 0; j < 32; ++j) xc[j * 16 * kXP] = c[j];
+      } else if (!PRUNE || (k2x == 1 && k1x < 16)) {   // the masked columns that pass B reads
 #pragma unroll
-        for (int j = 0; j < 32; ++j) xc[j * 4 * kXP] = make_float2(0.f, 0.f);
+        for (int j = 0; j < 32; ++j) xc[j * 16 * kXP] = make_float2(0.f, 0.f);
       }
       tc::fence_before();
       if (__syncthreads_or(bad)) goto abort;
@@ -1079,8 +1088,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_slice_tc(const SliceLaunch a, i
         constexpr int q = decltype(qq)::value;
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-          if constexpr (q != masked_k2x<false, PRUNE>()) b0[r * 4 + q] = xb[(128 * q + r) * kXP];
-          if constexpr (q != masked_k2x<true, PRUNE>()) b1[r * 4 + q] = xb[(128 * q + r) * kXP + 16];
+          if constexpr (q != masked_k2x<false, PRUNE>()) b0[r * 4 + q] = xb[(4 * x2_slot(q) + r) * kXP];
+          if constexpr (q != masked_k2x<true, PRUNE>()) b1[r * 4 + q] = xb[(4 * x2_slot(q) + r) * kXP + 16];
         }
       });
       passB_inv_tw<false, PRUNE>(b0, tB, twr[k1lo], twr[32 + k1lo]);
@@ -1089,10 +1098,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_slice_tc(const SliceLaunch a, i
       for (int q = 0; q < 4; ++q)
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
-          xb[(128 * q + r) * kXP] = b0[q * 4 + r];
-          xb[(128 * q + r) * kXP + 16] = b1[q * 4 + r];
+          xb[(4 * q + r) * kXP] = b0[q * 4 + r];
+          xb[(4 * q + r) * kXP + 16] = b1[q * 4 + r];
         }
-      __syncthreads();
+      __syncwarp();
       {
         const float4* const xa4r = reinterpret_cast<const float4*>(xa);
 #pragma unroll
