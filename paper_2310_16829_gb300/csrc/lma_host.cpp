@@ -1251,7 +1251,7 @@ lma_status slice_launch(lma_ctx* ctx, const lma_dev::SliceLaunch& L0, bool even,
     }
     float2* scratch = static_cast<float2*>(ctx->gen_scratch);
     ctx->tc_launched = true;   // the status word is checked at the next synchronizing read
-    CUDA_TRY(ctx, counted(ctx, K_SLICE, units, st, [&] { return lma_dev::launch_slice_gen(L, L.job[0].W, scratch, st); }));
+    CUDA_TRY(ctx, counted(ctx, K_SLICE, units, st, [&] { return lma_dev::launch_slice_gen(L, even, L.job[0].W, scratch, st); }));
     return LMA_OK;
   }
   if (prec == LMA_PREC_MIXED && ctx->rs_k1 == 0) {

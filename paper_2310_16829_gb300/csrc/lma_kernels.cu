@@ -66,6 +66,14 @@ __device__ __forceinline__ float2 psub(float2 a, float2 b) { return __ffma2_rn(b
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
   return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
+// a * b with its two roundings in stated places (the compiler is free to fuse either product of
+// cmul): which product is rounded before the FMA is part of a result's last bit
+__device__ __forceinline__ float2 cmul_yx(float2 a, float2 b) {
+  return make_float2(fmaf(a.x, b.x, -__fmul_rn(a.y, b.y)), fmaf(a.y, b.x, __fmul_rn(a.x, b.y)));
+}
+__device__ __forceinline__ float2 cmul_xy(float2 a, float2 b) {
+  return make_float2(fmaf(a.x, b.x, -__fmul_rn(a.y, b.y)), fmaf(a.x, b.y, __fmul_rn(a.y, b.x)));
+}
 // a * conj(b)
 __device__ __forceinline__ float2 cmulc(float2 a, float2 b) {
   return make_float2(a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y);
@@ -1477,29 +1485,47 @@ __global__ void __launch_bounds__(gen::kThreadsGen, 1) k_slice_256(const SliceLa
 }
 
 // ------------------------------------------------------------------------------------------
-// step a3 on W = 64 windows: each 64-point transform as two in-register 8-point passes
+// step a3 on W = 64 windows: whole 64-point rows and columns in the registers of one thread
 // ------------------------------------------------------------------------------------------
-// 64 = 8 x 8 as for W = 256: with x = 8 n + q and k = k1 + 8 k2, pass 1 takes the 8-point DFT
-// over n for residue q and multiplies by W_64^(q k1), pass 2 the DFT over q for k1; the
-// spectrum stays in digit-reversed order (entry 8 a + b holds frequency a + 8 b). The wave
-// (32 KiB) stays in shared memory in two buffers of opposite orientation, A[y][x] and
-// B[x][y] (rows of 65 entries). A phase reads one buffer with thread (c, g): c the position
-// along the other axis (the 32 lanes of a warp on consecutive positions), g = warp / 2 the
-// residue (pass 1) or k1 (pass 2); its passes work in place between CTA barriers, and it
-// writes its result transposed into the other buffer, so that the row phase runs the column
-// phase's code on B. Column phase: forward over y, propagator, inverse over y (A -> B). Row
-// phase: inverse over x, the next slice's transmission, forward over x (B -> A). The next
-// slice's transmission is staged into a third buffer by 8-byte cp.async while the column
-// phase runs. About 100 KB of shared memory: two CTAs per SM.
+// 64 = 8 x 8: with x = 8 n + q and k = k1 + 8 k2, pass 1 takes the 8-point DFT over n for each
+// residue q and multiplies by W_64^(q k1), pass 2 the DFT over q for each k1; frequency f sits
+// in register 8 (f % 8) + f / 8 between a forward and an inverse transform. A thread holds a
+// whole row (or column), so a slice crosses threads twice only: row spectra to columns and
+// back, through one shared buffer per wave of 64 rows x 66 entries. A CTA of 128 threads takes
+// two translates of one job: in the row phase thread (wave, y) runs inverse x, transmission,
+// forward x on its row; in the column phase a thread takes one live column (|kx| <= 21 with the
+// 2/3 bandlimit: 2 x 43 columns, so that one warp of four rests; which one rotates with the CTA,
+// to spread it over the SM's sub-partitions). Row accesses are 128-bit pairs (row pitch 33
+// 16-byte words: 8 lanes on 8 distinct slots), column accesses 64-bit on consecutive entries.
+// The next slice's transmission is staged by cp.async into the warp's own 32 rows once they
+// have been read.
+//
+// What bounds it: issue (57 % of cycles; 7,400 warp instructions per wave and slice) with 12 warps
+// per SM, limited by registers (64 complex values per thread); barrier and instruction-fetch
+// stalls. 16384 translates x 50 slices: 9.0 ms, against 14.5 ms with 8-point passes through
+// shared memory (k_slice_64_wide). The forward and the inverse transform appear once each in the
+// code (a loop over the two sides): with four copies the kernel waited for instructions (1.7
+// stall cycles per instruction, now 0.5) and took 9.9 ms.
 namespace w64 {
 constexpr int kN = 64;
-constexpr int kP = 65;                   // buffer row pitch (64-bit accesses of 16 lanes at stride 65 or 1: 32 banks)
-constexpr int kBufE = kN * kP;           // float2 per buffer
+constexpr int kWaves = 2;                // translates per CTA
+constexpr int kThreads64 = kWaves * kN;
+constexpr int kP = 66;                   // buffer row pitch
+constexpr int kWaveE = kN * kP;          // float2 per wave buffer
 // W_64^m = exp(-2 pi i m / 64), m < 64, built on the host in FP64 and rounded once
 __constant__ float2 c_tw[kN];
 
-// in-register 8-point DFT, natural order in and out: the first three stages of dft32
-template <bool INV>
+// bandlimit radius below 22: frequencies 22..42 are zero after the propagator
+constexpr int kNL = 43;                  // live frequencies per axis
+constexpr int kPR = 22;                  // propagator table row: |k| = 0..21
+__host__ __device__ constexpr bool live(int f) { return f <= 21 || f >= 43; }
+__host__ __device__ constexpr int freq(int c) { return c < 21 ? c + 43 : c - 21; }   // of column slot c
+__host__ __device__ constexpr int reg_of(int f) { return 8 * (f & 7) + (f >> 3); }
+__host__ __device__ constexpr int absf(int f) { return f <= 32 ? f : 64 - f; }
+
+// in-register 8-point DFT, natural order in and out: the first three stages of dft32. Bit i of
+// ZERO: input i is zero (never two that meet in the first stage); of SKIP: output i is not needed
+template <bool INV, int ZERO = 0, int SKIP = 0>
 __device__ __forceinline__ void dft8(float2 (&v)[8]) {
   float2 t[8];
   static_for<0, 8>([&](auto k) {
@@ -1512,7 +1538,13 @@ __device__ __forceinline__ void dft8(float2 (&v)[8]) {
       static_for<0, H>([&](auto j) {
         constexpr int I = decltype(blk)::value * 2 * H + decltype(j)::value;
         constexpr int M = decltype(j)::value * (16 / H);
-        bfly<INV, I, H, M>(t);
+        // first stage: t[I] = v[i0], t[I + 1] = v[i0 + 4]
+        constexpr int i0 = (I & 2) | ((I & 4) >> 2);
+        static_assert(H != 1 || !((ZERO >> i0) & (ZERO >> (i0 + 4)) & 1), "two zero inputs meet");
+        constexpr int Z = H != 1 ? 0 : ((ZERO >> i0) & 1 ? 1 : ((ZERO >> (i0 + 4)) & 1 ? 2 : 0));
+        constexpr bool NX = H != 4 || !((SKIP >> I) & 1);
+        constexpr bool NY = H != 4 || !((SKIP >> (I + 4)) & 1);
+        bfly<INV, I, H, M, NX, NY, Z>(t);
       });
     });
   });
@@ -1522,6 +1554,244 @@ __device__ __forceinline__ void dft8(float2 (&v)[8]) {
   });
 }
 
+// bits k2 of the masked frequencies k1 + 8 k2
+__host__ __device__ constexpr int masked_bits(int k1) {
+  int m = 0;
+  for (int k2 = 0; k2 < 8; ++k2)
+    if (!live(k1 + 8 * k2)) m |= 1 << k2;
+  return m;
+}
+
+// x natural in -> frequency f in v[reg_of(f)] (masked ones not formed)
+__device__ __forceinline__ void forward64(float2 (&v)[64]) {
+  static_for<0, 8>([&](auto qq) {
+    constexpr int q = decltype(qq)::value;
+    float2 a[8];
+#pragma unroll
+    for (int n = 0; n < 8; ++n) a[n] = v[8 * n + q];
+    dft8<false>(a);
+    v[q] = a[0];
+#pragma unroll
+    for (int k1 = 1; k1 < 8; ++k1) v[8 * k1 + q] = q == 0 ? a[k1] : cmul(a[k1], c_tw[q * k1]);
+  });
+  static_for<0, 8>([&](auto kk) {
+    constexpr int k1 = decltype(kk)::value;
+    float2 a[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) a[q] = v[8 * k1 + q];
+    dft8<false, 0, masked_bits(k1)>(a);
+#pragma unroll
+    for (int k2 = 0; k2 < 8; ++k2) v[8 * k1 + k2] = a[k2];
+  });
+}
+// frequency f in v[reg_of(f)] (masked ones taken as zero) -> x natural
+__device__ __forceinline__ void inverse64(float2 (&v)[64]) {
+  static_for<0, 8>([&](auto kk) {
+    constexpr int k1 = decltype(kk)::value;
+    float2 a[8];
+#pragma unroll
+    for (int k2 = 0; k2 < 8; ++k2) a[k2] = v[8 * k1 + k2];
+    dft8<true, masked_bits(k1), 0>(a);
+    v[8 * k1] = a[0];
+#pragma unroll
+    for (int q = 1; q < 8; ++q) v[8 * k1 + q] = k1 == 0 ? a[q] : cmulc(a[q], c_tw[k1 * q]);
+  });
+  static_for<0, 8>([&](auto qq) {
+    constexpr int q = decltype(qq)::value;
+    float2 a[8];
+#pragma unroll
+    for (int k1 = 0; k1 < 8; ++k1) a[k1] = v[8 * k1 + q];
+    dft8<true>(a);
+#pragma unroll
+    for (int n = 0; n < 8; ++n) v[8 * n + q] = a[n];
+  });
+}
+
+// 32 rows of 64 entries into a warp's buffer rows (asynchronous)
+template <bool EVEN>
+__device__ __forceinline__ void stage_rows(float2* rows, const float2* src, int pitch, int lane) {
+  if (EVEN) {
+#pragma unroll 8
+    for (int r = 0; r < 32; ++r) cp_async16(rows + r * kP + 2 * lane, src + static_cast<size_t>(r) * pitch + 2 * lane);
+  } else {
+#pragma unroll 8
+    for (int r = 0; r < 32; ++r) {
+      cp_async8(rows + r * kP + lane, src + static_cast<size_t>(r) * pitch + lane);
+      cp_async8(rows + r * kP + 32 + lane, src + static_cast<size_t>(r) * pitch + 32 + lane);
+    }
+  }
+  cp_async_commit();
+}
+constexpr int kSmemBytes = (kWaves * kWaveE + kPR * kPR) * 8;
+}  // namespace w64
+
+// Persistent CTAs (up to three per SM), complex64 exit waves, W = 64. Two translates of one job
+// per CTA; the last one of a job with an odd count is taken twice and stored once. EVEN: every
+// window origin of the list is even in x (16-byte staging).
+template <bool EVEN>
+__global__ void __launch_bounds__(w64::kThreads64, 3) k_slice_64(const SliceLaunch a, const int n_units) {
+  using namespace w64;
+  extern __shared__ __align__(16) float2 s64[];
+  float2* const ptab = s64 + kWaves * kWaveE;       // P[|ky|][|kx|], zero outside the bandlimit
+  const int T = threadIdx.x, lane = T & 31, warp = T >> 5;
+  // row role: row y of wave wr
+  const int wr = T >> 6, y = T & 63;
+  float2* const row = s64 + wr * kWaveE + y * kP;
+  float4* const row4 = reinterpret_cast<float4*>(row);
+  float2* const wrows = row - lane * kP;            // the warp's 32 rows
+  // column role: wave 0 has slots 0..42 at c = 0..42, wave 1 slots 11..42 at c = 43..74 and 0..10
+  // at c = 80..90, so that the two waves of a half-warp use distinct bank pairs
+  const int c = 32 * ((warp + blockIdx.x / max(1u, gridDim.x / 3)) & 3) + lane;
+  const int wc = c >= kNL, slot = c < kNL ? c : (c < 75 ? c - 32 : c - 80);
+  const bool col_live = c < 75 || (c >= 80 && c < 91);
+  const bool warp_live = __any_sync(0xffffffffu, col_live);   // lanes without a column transform values of no use
+  float2* const col = s64 + wc * kWaveE + slot;
+  const float2* const pcol = ptab + absf(freq(col_live ? slot : 0));
+  int cur_job = -1;
+  for (int u = blockIdx.x; u < n_units; u += gridDim.x) {
+    // unit u: items 2 u' and 2 u' + 1 of its job
+    int jb = 0, first = u;
+    while (true) {
+      const int n = (a.start[jb + 1] - a.start[jb] + 1) >> 1;
+      if (first < n) break;
+      first -= n;
+      ++jb;
+    }
+    const SliceJob& J = a.job[jb];
+    const int want = a.start[jb] + 2 * first + wr;
+    const int li = min(want, a.start[jb + 1] - 1);
+    const int n_slices = J.n_slices;
+    const int pitch = J.nx + kW;                          // padded transmission row
+    const size_t slice_elems = static_cast<size_t>(pitch) * (J.ny + kW);
+    const int item = a.list[li];
+    const int cfg = item / J.n_translates;
+    const int ti = item - cfg * J.n_translates;
+    const int ia = ti % J.lat_nax, ib = ti / J.lat_nax;
+    int ox = (J.lat_ox + ia * J.lat_sx - kN / 2) % J.nx;
+    if (ox < 0) ox += J.nx;
+    int oy = (J.lat_oy + ib * J.lat_sy - kN / 2) % J.ny;
+    if (oy < 0) oy += J.ny;
+    // the halo of kW >= 64 pixels keeps every window inside the padded array
+    const float2* tsrc = J.t + cfg * J.t_slot + static_cast<size_t>(oy + (y & 32)) * pitch + ox;
+    const int oi = a.out_index ? a.out_index[li] : ti;
+    float2 v[64];
+    auto load_row = [&]() {
+#pragma unroll
+      for (int x = 0; x < 64; x += 2) {
+        const float4 p = row4[x / 2];
+        v[x] = make_float2(p.x, p.y);
+        v[x + 1] = make_float2(p.z, p.w);
+      }
+    };
+    __syncwarp();   // the previous item's store has read the rows
+    stage_rows<true>(wrows, J.uW + (y & 32) * kN, kN, lane);
+    if (jb != cur_job) {
+      // the previous item's last barrier is past every read of the table; the barrier after the
+      // first forward transform publishes it
+      cur_job = jb;
+      for (int e = T; e < kPR * kPR; e += kThreads64) {
+        const int pb = e / kPR, pa = e - pb * kPR;
+        ptab[e] = pa * pa + pb * pb <= J.r2max ? cmul_yx(J.ex[pa], J.ey[pb]) : make_float2(0.f, 0.f);
+      }
+    }
+    cp_async_wait_all();
+    __syncwarp();
+    load_row();
+    __syncwarp();
+    if (n_slices > 0) stage_rows<EVEN>(wrows, tsrc, pitch, lane);
+    for (int s = 0; s < n_slices; ++s) {
+      // forward over x on rows (side 0), then over y on columns (side 1): one copy of the
+      // transform's code for both
+#pragma unroll 1
+      for (int side = 0; side < 2; ++side) {
+        if (side == 0) {
+          // transmission of slice s
+          cp_async_wait_all();
+          __syncwarp();
+#pragma unroll
+          for (int x = 0; x < 64; x += 2) {
+            const float4 p = row4[x / 2];
+            v[x] = cmul_yx(v[x], make_float2(p.x, p.y));
+            v[x + 1] = cmul_yx(v[x + 1], make_float2(p.z, p.w));
+          }
+        } else if (col_live) {
+#pragma unroll
+          for (int k = 0; k < 64; ++k) v[k] = col[k * kP];
+        }
+        if (side == 0 || warp_live) forward64(v);
+        if (side == 0) {
+          // the live entries go to the row's slots
+          static_for<0, kNL / 2>([&](auto cc) {
+            constexpr int C = 2 * decltype(cc)::value;
+            const float2 p = v[reg_of(freq(C))], q = v[reg_of(freq(C + 1))];
+            row4[C / 2] = make_float4(p.x, p.y, q.x, q.y);
+          });
+          if constexpr (kNL & 1) row[kNL - 1] = v[reg_of(freq(kNL - 1))];
+          __syncthreads();
+        } else if (col_live) {
+          // propagation (Sec. 3.2)
+          static_for<0, 64>([&](auto ff) {
+            constexpr int F = decltype(ff)::value;
+            if constexpr (live(F)) v[reg_of(F)] = cmul_xy(v[reg_of(F)], pcol[absf(F) * kPR]);
+          });
+        }
+      }
+      // inverse over y on columns, then over x on rows
+#pragma unroll 1
+      for (int side = 1; side >= 0; --side) {
+        if (side == 0 || warp_live) inverse64(v);
+        if (side == 1) {
+          if (col_live) {
+#pragma unroll
+            for (int k = 0; k < 64; ++k) col[k * kP] = v[k];
+          }
+          __syncthreads();
+          static_for<0, kNL / 2>([&](auto cc) {
+            constexpr int C = 2 * decltype(cc)::value;
+            const float4 p = row4[C / 2];
+            v[reg_of(freq(C))] = make_float2(p.x, p.y);
+            v[reg_of(freq(C + 1))] = make_float2(p.z, p.w);
+          });
+          if constexpr (kNL & 1) v[reg_of(freq(kNL - 1))] = row[kNL - 1];
+          __syncwarp();
+          if (s + 1 < n_slices) {
+            tsrc += slice_elems;
+            stage_rows<EVEN>(wrows, tsrc, pitch, lane);
+          }
+        }
+      }
+    }
+    // the exit wave leaves through the warp's rows: 512 contiguous bytes per store instruction
+#pragma unroll
+    for (int x = 0; x < 64; x += 2) row4[x / 2] = make_float4(v[x].x, v[x].y, v[x + 1].x, v[x + 1].y);
+    __syncwarp();
+    if (want == li) {
+      float4* const dst = reinterpret_cast<float4*>(J.U + cfg * J.u_slot + static_cast<size_t>(oi) * (kN * kN) + (y & 32) * kN);
+#pragma unroll 8
+      for (int r = 0; r < 32; ++r) dst[r * (kN / 2) + lane] = *reinterpret_cast<const float4*>(wrows + r * kP + 2 * lane);
+    }
+  }
+}
+
+// The same with 512 threads per translate and any bandlimit: each 64-point transform as two 8-point
+// passes through shared memory, 8 values per thread. It serves the lists that give every translate
+// an SM of its own (PER_SM = 1: 32 to 77 translates x 50 slices take 140 us, 253 us in k_slice_64,
+// which runs an eighth of the warps per translate; at 165 translates the two take 262 us each),
+// and bandlimit radii from 22 pixels (PER_SM = 2), where k_slice_64 would have 64 columns and more
+// registers than threads can hold (k_slice_64 written for them: 877 us against 800 at 837
+// translates, 3.15 ms against 3.68 at 4096). The wave (32 KiB) stays in two buffers of opposite
+// orientation, A[y][x] and B[x][y] (rows of 65 entries). A phase reads one buffer with thread
+// (c, g): c the position along the other axis (the 32 lanes of a warp on consecutive positions),
+// g = warp / 2 the residue (pass 1) or k1 (pass 2); its passes work in place between CTA
+// barriers, and it writes its result transposed into the other buffer, so that the row phase runs
+// the column phase's code on B. The next slice's transmission is staged into a third buffer by
+// 8-byte cp.async while the column phase runs.
+namespace w64w {
+using w64::c_tw;
+using w64::dft8;
+using w64::kN;
+constexpr int kP = 65;                   // buffer row pitch (64-bit accesses of 16 lanes at stride 65 or 1: 32 banks)
+constexpr int kBufE = kN * kP;           // float2 per buffer
 // forward over one axis for thread (c, g) of buffer X: pass 1 from v[n] = x[8 n + g] (already
 // in registers), pass 2; X[entry][c] is the in-place scratch; v[k2] = X[g + 8 k2] after it
 __device__ __forceinline__ void forward(float2* X, float2 (&v)[8], int c, int g) {
@@ -1548,11 +1818,12 @@ __device__ __forceinline__ void inverse(float2* X, float2 (&v)[8], int c, int g)
   for (int k1 = 0; k1 < 8; ++k1) v[k1] = X[(8 * k1 + g) * kP + c];
   dft8<true>(v);
 }
-}  // namespace w64
+constexpr int kSmemBytes = (3 * kBufE + kN) * 8;   // A, B, staged transmission, ey
+}  // namespace w64w
 
-// One translate per CTA at a time (persistent CTAs, two per SM), complex64 exit waves, W = 64.
-__global__ void __launch_bounds__(512, 2) k_slice_64(const SliceLaunch a) {
-  using namespace w64;
+template <int PER_SM>
+__global__ void __launch_bounds__(512, PER_SM) k_slice_64_wide(const SliceLaunch a) {
+  using namespace w64w;
   extern __shared__ __align__(16) float2 s64[];
   float2* const A = s64;                 // A[y][x entry]
   float2* const B = A + kBufE;           // B[x][y]
@@ -1606,7 +1877,7 @@ __global__ void __launch_bounds__(512, 2) k_slice_64(const SliceLaunch a) {
       // rows y = c: the input wave times the transmission of slice 0, forward over x into A
       float2 v[8];
 #pragma unroll
-      for (int n = 0; n < 8; ++n) v[n] = cmul(J.uW[c * kN + 8 * n + g], Tb[c * kP + 8 * n + g]);
+      for (int n = 0; n < 8; ++n) v[n] = cmul_yx(J.uW[c * kN + 8 * n + g], Tb[c * kP + 8 * n + g]);
       forward(B, v, c, g);
 #pragma unroll
       for (int k2 = 0; k2 < 8; ++k2) A[c * kP + 8 * g + k2] = v[k2];
@@ -1628,7 +1899,7 @@ __global__ void __launch_bounds__(512, 2) k_slice_64(const SliceLaunch a) {
         for (int k2 = 0; k2 < 8; ++k2) {
           const int kyi = g + 8 * k2;
           const int kys = kyi < kN / 2 ? kyi : kyi - kN;
-          v[k2] = kxs * kxs + kys * kys <= J.r2max ? cmul(v[k2], cmul(ex, eyt[kyi])) : make_float2(0.f, 0.f);
+          v[k2] = kxs * kxs + kys * kys <= J.r2max ? cmul_xy(v[k2], cmul_yx(ex, eyt[kyi])) : make_float2(0.f, 0.f);
         }
         inverse(A, v, c, g);
 #pragma unroll
@@ -1644,7 +1915,7 @@ __global__ void __launch_bounds__(512, 2) k_slice_64(const SliceLaunch a) {
         inverse(B, v, c, g);
         if (s + 1 < n_slices) {
 #pragma unroll
-          for (int n = 0; n < 8; ++n) v[n] = cmul(v[n], Tb[c * kP + 8 * n + g]);
+          for (int n = 0; n < 8; ++n) v[n] = cmul_yx(v[n], Tb[c * kP + 8 * n + g]);
           forward(B, v, c, g);
 #pragma unroll
           for (int k2 = 0; k2 < 8; ++k2) A[c * kP + 8 * g + k2] = v[k2];
@@ -2591,10 +2862,9 @@ cudaError_t noalloc_scratch(void** ptr) {
 size_t slice_smem_bytes() { return static_cast<size_t>(kSliceSmemFloat2) * sizeof(float2); }
 size_t synth_smem_bytes() { return static_cast<size_t>(kSynthSmemFloat2) * sizeof(float2); }
 size_t slice_tc_smem_bytes() { return static_cast<size_t>(kSliceTcSmemBytes); }
-static size_t slice_gen_smem_bytes(int W) {
-  return W <= 64 ? (3 * static_cast<size_t>(w64::kBufE) + w64::kN) * sizeof(float2)   // A, B, staged t, ey
-                 : (2 * static_cast<size_t>(w256::kBuf) + w256::kN) * sizeof(float2) +
-                       (2 + 2 * gen::kThreadsGen / 32) * sizeof(uint64_t);   // two panel buffers, ey, mbarriers
+static size_t slice_256_smem_bytes() {
+  return (2 * static_cast<size_t>(w256::kBuf) + w256::kN) * sizeof(float2) +
+         (2 + 2 * gen::kThreadsGen / 32) * sizeof(uint64_t);   // two panel buffers, ey, mbarriers
 }
 cudaError_t launch_selftest_wait(int which, int* status, cudaStream_t s) {
   k_selftest_wait<<<1, which == 0 ? 32 : gen::kThreadsGen, 0, s>>>(status);
@@ -2681,15 +2951,16 @@ cudaError_t init_device_constants() {
     for (int m = 0; m < w64::kN; ++m)
       tw1[m] = make_float2(static_cast<float>(cos(-2.0 * pi * m / 64)), static_cast<float>(sin(-2.0 * pi * m / 64)));
     if ((e = cudaMemcpyToSymbol(w64::c_tw, tw1, sizeof(tw1))) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_slice_64, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  static_cast<int>(slice_gen_smem_bytes(64)))) != cudaSuccess)
-      return e;
+    for (auto f : {k_slice_64_wide<1>, k_slice_64_wide<2>})
+      if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, w64w::kSmemBytes)) != cudaSuccess) return e;
+    for (auto f : {k_slice_64<false>, k_slice_64<true>})
+      if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, w64::kSmemBytes)) != cudaSuccess) return e;
     float2 tw2[w256::kN];
     for (int m = 0; m < w256::kN; ++m)
       tw2[m] = make_float2(static_cast<float>(cos(-2.0 * pi * m / 256)), static_cast<float>(sin(-2.0 * pi * m / 256)));
     if ((e = cudaMemcpyToSymbol(w256::c_tw, tw2, sizeof(tw2))) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(k_slice_256, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  static_cast<int>(slice_gen_smem_bytes(256)))) != cudaSuccess)
+                                  static_cast<int>(slice_256_smem_bytes()))) != cudaSuccess)
       return e;
   }
   const int sr = static_cast<int>(slice_rs_smem_bytes());
@@ -2774,19 +3045,29 @@ cudaError_t launch_slice_tc(const SliceLaunch& a, bool even_origins, cudaStream_
   return cudaGetLastError();
 }
 
-cudaError_t launch_slice_gen(const SliceLaunch& a, int W, float2* scratch, cudaStream_t s) {
+cudaError_t launch_slice_gen(const SliceLaunch& a, bool even_origins, int W, float2* scratch, cudaStream_t s) {
   if (a.n_list <= 0) return cudaSuccess;
   if (a.n_jobs < 1 || a.n_jobs > kMaxJobs || a.start[0] != 0 || a.start[a.n_jobs] != a.n_list || !a.status)
     return cudaErrorInvalidValue;
   // persistent, one CTA per SM: W = 256 takes one scratch wave per CTA
   const int grid = a.n_list < sm_count() ? a.n_list : sm_count();
   if (W == 64) {
-    // two CTAs per SM
-    const int grid64 = a.n_list < 2 * sm_count() ? a.n_list : 2 * sm_count();
-    k_slice_64<<<grid64, 512, slice_gen_smem_bytes(64), s>>>(a);
+    bool prune = true;   // k_slice_64 needs every job's bandlimit radius below 22 pixels
+    int units = 0;       // its CTAs take two translates of one job
+    for (int i = 0; i < a.n_jobs; ++i) {
+      units += (a.start[i + 1] - a.start[i] + 1) / 2;
+      prune = prune && a.job[i].r2max < 22 * 22;
+    }
+    const int sms = sm_count();
+    if (a.n_list <= sms)
+      k_slice_64_wide<1><<<a.n_list, 512, w64w::kSmemBytes, s>>>(a);
+    else if (!prune)
+      k_slice_64_wide<2><<<a.n_list < 2 * sms ? a.n_list : 2 * sms, 512, w64w::kSmemBytes, s>>>(a);
+    else
+      (even_origins ? k_slice_64<true> : k_slice_64<false>)<<<units < 3 * sms ? units : 3 * sms, w64::kThreads64, w64::kSmemBytes, s>>>(a, units);
   } else if (W == 256) {
     if (!scratch) return cudaErrorInvalidValue;
-    k_slice_256<<<grid, gen::kThreadsGen, slice_gen_smem_bytes(256), s>>>(a, scratch, a.status);
+    k_slice_256<<<grid, gen::kThreadsGen, slice_256_smem_bytes(), s>>>(a, scratch, a.status);
   } else {
     return cudaErrorInvalidValue;
   }
