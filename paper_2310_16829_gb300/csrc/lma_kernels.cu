@@ -78,6 +78,9 @@ __device__ __forceinline__ float2 cmul_xy(float2 a, float2 b) {
 __device__ __forceinline__ float2 cmulc(float2 a, float2 b) {
   return make_float2(a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y);
 }
+__device__ __forceinline__ float2 cmulc_y(float2 a, float2 b) {   // the products with b.y are rounded first
+  return make_float2(fmaf(a.x, b.x, __fmul_rn(a.y, b.y)), fmaf(a.y, b.x, -__fmul_rn(a.x, b.y)));
+}
 __device__ __forceinline__ float2 cfma(float2 acc, float2 a, float2 b) {
   return make_float2(fmaf(a.x, b.x, fmaf(-a.y, b.y, acc.x)), fmaf(a.x, b.y, fmaf(a.y, b.x, acc.y)));
 }
@@ -218,7 +221,9 @@ __device__ __forceinline__ void dft32(float2 (&v)[32]) {
 // In-register 16-point DFT, natural order in and out: the first four stages of dft32 on 16
 // values (W_16^m = W_32^(2m), so stage H takes the twiddle index j (16 / H) of dft32)
 __host__ __device__ constexpr int brev4(int k) { return ((k & 1) << 3) | ((k & 2) << 1) | ((k & 4) >> 1) | ((k & 8) >> 3); }
-template <bool INV>
+// Bit i of ZERO: input i is zero (never two that meet in the first stage); of SKIP: output i is
+// not needed.
+template <bool INV, int ZERO = 0, int SKIP = 0>
 __device__ __forceinline__ void dft16(float2 (&v)[16]) {
   float2 t[16];
   static_for<0, 16>([&](auto k) {
@@ -231,7 +236,13 @@ __device__ __forceinline__ void dft16(float2 (&v)[16]) {
       static_for<0, H>([&](auto j) {
         constexpr int I = decltype(blk)::value * 2 * H + decltype(j)::value;
         constexpr int M = decltype(j)::value * (16 / H);
-        bfly<INV, I, H, M>(t);
+        // first stage: t[I] = v[i0], t[I + 1] = v[i0 + 8]
+        constexpr int i0 = brev4(I & 14);
+        static_assert(H != 1 || !((ZERO >> i0) & (ZERO >> (i0 + 8)) & 1), "two zero inputs meet");
+        constexpr int Z = H != 1 ? 0 : ((ZERO >> i0) & 1 ? 1 : ((ZERO >> (i0 + 8)) & 1 ? 2 : 0));
+        constexpr bool NX = H != 8 || !((SKIP >> I) & 1);
+        constexpr bool NY = H != 8 || !((SKIP >> ((I + 8) & 15)) & 1);
+        bfly<INV, I, H, M, NX, NY, Z>(t);
       });
     });
   });
@@ -1322,7 +1333,7 @@ __device__ __forceinline__ void row_inverse(float2* row, float2 (&v)[16], int j,
 // two row slots on its own two mbarriers, so the row phase has no CTA barrier. Every wait is
 // one polling lane per warp (bounded, suspended tries) and then one try_wait per lane. Scratch
 // copies carry an evict-last L2 policy; the exit wave is written with streaming stores.
-__global__ void __launch_bounds__(gen::kThreadsGen, 1) k_slice_256(const SliceLaunch a, float2* scratch, int* status) {
+__global__ void __launch_bounds__(gen::kThreadsGen, 1) k_slice_256_any(const SliceLaunch a, float2* scratch, int* status) {
   using namespace w256;
   extern __shared__ __align__(16) unsigned char smg[];
   float2* const S = reinterpret_cast<float2*>(smg);
@@ -1484,6 +1495,241 @@ __global__ void __launch_bounds__(gen::kThreadsGen, 1) k_slice_256(const SliceLa
   if (bad && T == 0) atomicOr(status, 1);
 }
 
+// The same transforms for bandlimit radii up to 85 pixels (2/3 of Nyquist is 85.3), without panels
+// and without barriers inside a phase. Frequencies 88..167 are zero after the propagator: of the
+// 16 k2 of a pass-2 thread 5 are dead (k2 = 6..10 for k1 < 8, 5..9 for k1 >= 8), so only 44 of 64
+// groups of 4 columns are transformed over y, stored and read.
+//   A warp's task is 4 rows (row phase) or 4 columns (column phase); lane (a, j) = (lane / 8, lane
+//   % 8) holds of row or column a the residues (pass 2: the k1) j and j + 8, 32 values in
+//   registers, and both passes of a transform exchange through the warp's own 4 x 264 entries
+//   (entry 16 k1 + q at 16 k1 + (q ^ k1), rows 264 apart: every access of a half-warp falls on 16
+//   distinct bank pairs), so the only CTA barriers are the two between the phases of a slice.
+//   The scratch holds column groups [44][256 rows][4]: a column task loads and stores 256
+//   contiguous bytes per instruction, a row task two runs of 128.
+//   The transmission of a row task is staged by cp.async into the warp's entries while the
+//   inverse's last pass runs. The window's halves x, y < 128 and >= 128 have their own origins in
+//   the padded array (halo of 128 pixels), so that no index wraps.
+//   The propagator is a shared table over |ky|, |kx| <= 88, zero outside the bandlimit (rows of 90
+//   entries: 8 consecutive ky and 2 kx of a half-warp on 16 bank pairs).
+//
+// What bounds it: the shared-memory and L1 pipe (85 % of cycles: exchanges, twiddles, scratch and
+// staging; issue 50 %, FP32 pipe 43 %). 4096 translates x 20 slices: 24.6 ms, against 39.5 ms in
+// k_slice_256_any (half of its instructions and about two thirds of its scratch traffic).
+namespace w256p {
+using w256::kN;
+constexpr int kPitch = 264;              // exchange row
+constexpr int kWarpE = 4 * kPitch;
+constexpr int kGroups = 44;              // column groups of 4: frequencies 0..87, 168..255
+constexpr int kScratchE = kGroups * kN * 4;   // float2 per CTA
+constexpr int kR = 88;                   // largest |k| of a column group
+constexpr int kPR = 90;                  // propagator table row
+constexpr int kSmemBytes = (16 * kWarpE + 256 + (kR + 1) * kPR) * 8;
+// masked k2 of the two k1 of a lane (j and j + 8)
+constexpr int kMask0 = 0x7c0, kMask1 = 0x3e0;
+__host__ __device__ constexpr bool live(int h, int k2) { return !(((h ? kMask1 : kMask0) >> k2) & 1); }
+// first column group (of 4 frequencies) of frequencies 16 k2 + 8 h + 0..7
+__host__ __device__ constexpr int group(int h, int k2) { return k2 < 8 ? 4 * k2 + 2 * h : 4 * k2 + 2 * h - 20; }
+__device__ __forceinline__ int absk(int f) { return f < kN / 2 ? f : kN - f; }
+
+// forward of a warp's 4 rows or columns: v[h][n] = x[16 n + j + 8 h] -> v[h][k2] = X[j + 8 h + 16 k2]
+// (masked ones not formed); ex: the warp's entries + a * kPitch; tw: W_256^(jj m) at entry
+// ((m / 2) * 16 + jj) * 2 + m % 2
+__device__ __forceinline__ void forward(float2 (&v)[2][16], float2* ex, const float4* tw, int j) {
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    dft16<false>(v[h]);
+#pragma unroll
+    for (int m = 0; m < 16; m += 2) {
+      const float4 w = tw[(m / 2) * 16 + j + 8 * h];
+      if (m > 0) v[h][m] = cmul_yx(v[h][m], make_float2(w.x, w.y));
+      v[h][m + 1] = cmul_yx(v[h][m + 1], make_float2(w.z, w.w));
+    }
+#pragma unroll
+    for (int k1 = 0; k1 < 16; ++k1) ex[16 * k1 + ((j + 8 * h) ^ k1)] = v[h][k1];
+  }
+  __syncwarp();
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int k1 = j + 8 * h;
+#pragma unroll
+    for (int q = 0; q < 16; ++q) v[h][q] = ex[16 * k1 + (q ^ k1)];
+  }
+  dft16<false, 0, kMask0>(v[0]);
+  dft16<false, 0, kMask1>(v[1]);
+}
+// inverse, first pass and exchange: v[h][k2] = X[j + 8 h + 16 k2] (masked ones taken as zero) ->
+// v[h][k1] before the last 16-point pass over k1, for residue q = j + 8 h
+__device__ __forceinline__ void inverse_exchange(float2 (&v)[2][16], float2* ex, const float4* tw, int j) {
+  dft16<true, kMask0, 0>(v[0]);
+  dft16<true, kMask1, 0>(v[1]);
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int k1 = j + 8 * h;
+#pragma unroll
+    for (int m = 0; m < 16; m += 2) {
+      const float4 w = tw[(m / 2) * 16 + k1];
+      if (m > 0) v[h][m] = cmulc_y(v[h][m], make_float2(w.x, w.y));
+      v[h][m + 1] = cmulc_y(v[h][m + 1], make_float2(w.z, w.w));
+    }
+#pragma unroll
+    for (int q = 0; q < 16; ++q) ex[16 * k1 + (q ^ k1)] = v[h][q];
+  }
+  __syncwarp();
+#pragma unroll
+  for (int h = 0; h < 2; ++h)
+#pragma unroll
+    for (int k1 = 0; k1 < 16; ++k1) v[h][k1] = ex[16 * k1 + ((j + 8 * h) ^ k1)];
+  __syncwarp();   // the entries are free again
+}
+}  // namespace w256p
+
+// One translate per CTA at a time (persistent CTAs, one per SM), complex64 exit waves; scratch:
+// w256p::kScratchE complex64 per CTA. EVEN: every window origin of the list is even in x.
+template <bool EVEN>
+__global__ void __launch_bounds__(512, 1) k_slice_256(const SliceLaunch a, float2* scratch) {
+  using namespace w256p;
+  extern __shared__ __align__(16) float2 s256[];
+  const int T = threadIdx.x, warp = T >> 5, lane = T & 31;
+  const int ra = lane >> 3, j = lane & 7;           // row or column of the task, residue (and + 8)
+  float2* const wx = s256 + warp * kWarpE;
+  float2* const ex = wx + ra * kPitch;
+  float2* const twt = s256 + 16 * kWarpE;
+  const float4* const tw = reinterpret_cast<const float4*>(twt);
+  float2* const ptab = twt + 256;
+  float2* const G = scratch + static_cast<size_t>(blockIdx.x) * kScratchE;
+  if (T < 256) twt[((T >> 1 & 7) * 16 + (T >> 4)) * 2 + (T & 1)] = w256::c_tw[(T >> 4) * (T & 15)];
+  int cur_job = -1;
+  for (int li = blockIdx.x; li < a.n_list; li += gridDim.x) {
+    int jb = 0;
+    while (jb + 1 < a.n_jobs && li >= a.start[jb + 1]) ++jb;
+    const SliceJob& J = a.job[jb];
+    const int n_slices = J.n_slices;
+    const int pitch = J.nx + kW;                          // padded transmission row
+    const size_t slice_elems = static_cast<size_t>(pitch) * (J.ny + kW);
+    const int item = a.list[li];
+    const int cfg = item / J.n_translates;
+    const int ti = item - cfg * J.n_translates;
+    const int ia = ti % J.lat_nax, ib = ti / J.lat_nax;
+    int ox = (J.lat_ox + ia * J.lat_sx - kN / 2) % J.nx;
+    if (ox < 0) ox += J.nx;
+    int oy = (J.lat_oy + ib * J.lat_sy - kN / 2) % J.ny;
+    if (oy < 0) oy += J.ny;
+    // origins of the window's right and lower halves
+    const int ox2 = ox + kW >= J.nx ? ox + kW - J.nx : ox + kW, oy2 = oy + kW >= J.ny ? oy + kW - J.ny : oy + kW;
+    const float2* const tbase = J.t + cfg * J.t_slot;
+    const int oi = a.out_index ? a.out_index[li] : ti;
+    float2* const ud = J.U + cfg * J.u_slot + static_cast<size_t>(oi) * (kN * kN);
+    if (jb != cur_job) {
+      cur_job = jb;
+      __syncthreads();   // the previous item's reads of the table are over
+      for (int e = T; e < (kR + 1) * kPR; e += 512) {
+        const int pb = e / kPR, pa = e - pb * kPR;
+        ptab[e] = pa <= kR && pa * pa + pb * pb <= J.r2max ? cmul_yx(J.ex[pa], J.ey[pb]) : make_float2(0.f, 0.f);
+      }
+    }
+    __syncthreads();     // twiddles, the propagator table; the previous item's scratch rows are read
+    for (int s = -1; s < n_slices; ++s) {
+      if (s >= 0) {
+        // columns: forward over y, propagation (Sec. 3.2), inverse over y
+        for (int g = warp; g < kGroups; g += 16) {
+          float2* const col = G + g * (kN * 4) + j * 4 + ra;   // row y at + 4 y
+          float2 v[2][16];
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int n = 0; n < 16; ++n) v[h][n] = __ldcg(col + 4 * (16 * n + 8 * h));
+          forward(v, ex, tw, j);
+          const float2* const pc = ptab + absk((g < kGroups / 2 ? 4 * g : 4 * g + 80) + ra);
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            static_for<0, 16>([&](auto kk) {
+              constexpr int k2 = decltype(kk)::value;
+              if (live(h, k2)) v[h][k2] = cmul_xy(v[h][k2], pc[absk(16 * k2 + 8 * h + j) * kPR]);
+            });
+          __syncwarp();   // every lane has read its entries of the forward exchange
+          inverse_exchange(v, ex, tw, j);
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            dft16<true>(v[h]);
+#pragma unroll
+            for (int n = 0; n < 16; ++n) __stcg(col + 4 * (16 * n + 8 * h), v[h][n]);
+          }
+        }
+        __syncthreads();
+      }
+      // rows: inverse over x (the input wave first), the next slice's transmission, forward over x
+      const bool last = s + 1 == n_slices;   // rows go to the exit wave, not back
+      for (int q = warp; q < kN / 4; q += 16) {
+        const int y = 4 * q + ra;
+        float2* const row = G + y * 4 + (j >> 2) * (kN * 4) + (j & 3);   // frequencies 16 k2 + 8 h + j at + group(h, k2) * 1024
+        float2 v[2][16];
+        if (s >= 0) {
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            static_for<0, 16>([&](auto kk) {
+              constexpr int k2 = decltype(kk)::value;
+              if (live(h, k2)) v[h][k2] = __ldcg(row + group(h, k2) * (kN * 4));
+            });
+          inverse_exchange(v, ex, tw, j);
+        } else {
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int n = 0; n < 16; ++n) v[h][n] = J.uW[y * kN + 16 * n + 8 * h + j];
+        }
+        if (!last) {
+          // four rows of transmission into the warp's entries
+          const float2* const src = tbase + (s + 1) * slice_elems + static_cast<size_t>(q < kN / 8 ? oy + 4 * q : oy2 + 4 * q - kW) * pitch;
+#pragma unroll
+          for (int r = 0; r < 4; ++r) {
+            const float2* const t0 = src + static_cast<size_t>(r) * pitch;
+            if (EVEN) {
+              cp_async16(wx + r * kPitch + 2 * lane, t0 + ox + 2 * lane);
+              cp_async16(wx + r * kPitch + 64 + 2 * lane, t0 + ox + 64 + 2 * lane);
+              cp_async16(wx + r * kPitch + 128 + 2 * lane, t0 + ox2 + 2 * lane);
+              cp_async16(wx + r * kPitch + 192 + 2 * lane, t0 + ox2 + 64 + 2 * lane);
+            } else {
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                cp_async8(wx + r * kPitch + 32 * i + lane, t0 + ox + 32 * i + lane);
+                cp_async8(wx + r * kPitch + 128 + 32 * i + lane, t0 + ox2 + 32 * i + lane);
+              }
+            }
+          }
+          cp_async_commit();
+        }
+        if (s >= 0) {
+          dft16<true>(v[0]);
+          dft16<true>(v[1]);
+        }
+        if (last) {
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int n = 0; n < 16; ++n) __stcs(ud + y * kN + 16 * n + 8 * h + j, v[h][n]);
+        } else {
+          cp_async_wait_all();
+          __syncwarp();
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int n = 0; n < 16; ++n) v[h][n] = cmul_yx(v[h][n], ex[16 * n + 8 * h + j]);
+          __syncwarp();   // every lane has read its transmission
+          forward(v, ex, tw, j);
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            static_for<0, 16>([&](auto kk) {
+              constexpr int k2 = decltype(kk)::value;
+              if (live(h, k2)) __stcg(row + group(h, k2) * (kN * 4), v[h][k2]);
+            });
+          __syncwarp();   // the forward exchange is read
+        }
+      }
+      __syncthreads();
+    }
+  }
+}
+
 // ------------------------------------------------------------------------------------------
 // step a3 on W = 64 windows: whole 64-point rows and columns in the registers of one thread
 // ------------------------------------------------------------------------------------------
@@ -1572,7 +1818,7 @@ __device__ __forceinline__ void forward64(float2 (&v)[64]) {
     dft8<false>(a);
     v[q] = a[0];
 #pragma unroll
-    for (int k1 = 1; k1 < 8; ++k1) v[8 * k1 + q] = q == 0 ? a[k1] : cmul(a[k1], c_tw[q * k1]);
+    for (int k1 = 1; k1 < 8; ++k1) v[8 * k1 + q] = q == 0 ? a[k1] : cmul_yx(a[k1], c_tw[q * k1]);
   });
   static_for<0, 8>([&](auto kk) {
     constexpr int k1 = decltype(kk)::value;
@@ -1594,7 +1840,7 @@ __device__ __forceinline__ void inverse64(float2 (&v)[64]) {
     dft8<true, masked_bits(k1), 0>(a);
     v[8 * k1] = a[0];
 #pragma unroll
-    for (int q = 1; q < 8; ++q) v[8 * k1 + q] = k1 == 0 ? a[q] : cmulc(a[q], c_tw[k1 * q]);
+    for (int q = 1; q < 8; ++q) v[8 * k1 + q] = k1 == 0 ? a[q] : cmulc_y(a[q], c_tw[k1 * q]);
   });
   static_for<0, 8>([&](auto qq) {
     constexpr int q = decltype(qq)::value;
@@ -2959,7 +3205,9 @@ cudaError_t init_device_constants() {
     for (int m = 0; m < w256::kN; ++m)
       tw2[m] = make_float2(static_cast<float>(cos(-2.0 * pi * m / 256)), static_cast<float>(sin(-2.0 * pi * m / 256)));
     if ((e = cudaMemcpyToSymbol(w256::c_tw, tw2, sizeof(tw2))) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_slice_256, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    for (auto f : {k_slice_256<false>, k_slice_256<true>})
+      if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, w256p::kSmemBytes)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(k_slice_256_any, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   static_cast<int>(slice_256_smem_bytes()))) != cudaSuccess)
       return e;
   }
@@ -3067,7 +3315,12 @@ cudaError_t launch_slice_gen(const SliceLaunch& a, bool even_origins, int W, flo
       (even_origins ? k_slice_64<true> : k_slice_64<false>)<<<units < 3 * sms ? units : 3 * sms, w64::kThreads64, w64::kSmemBytes, s>>>(a, units);
   } else if (W == 256) {
     if (!scratch) return cudaErrorInvalidValue;
-    k_slice_256<<<grid, gen::kThreadsGen, slice_256_smem_bytes(), s>>>(a, scratch, a.status);
+bool prune = true;   // k_slice_256 needs every job's bandlimit radius below 86 pixels
+    for (int i = 0; i < a.n_jobs; ++i) prune = prune && a.job[i].r2max < 86 * 86;
+    if (prune)
+      (even_origins ? k_slice_256<true> : k_slice_256<false>)<<<grid, 512, w256p::kSmemBytes, s>>>(a, scratch);
+    else
+      k_slice_256_any<<<grid, gen::kThreadsGen, slice_256_smem_bytes(), s>>>(a, scratch, a.status);
   } else {
     return cudaErrorInvalidValue;
   }
