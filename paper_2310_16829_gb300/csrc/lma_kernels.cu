@@ -2534,27 +2534,48 @@ __global__ void __launch_bounds__(kThreads, 1) k_synth_detect(const SynthArgs a)
           acc[2 * b + 1] = cfma2(acc[2 * b + 1], al4, f1);
         }
       } else {
+        // an odd placement breaks the pairs: each column by itself, in two rounds of 4 rows whose
+        // 16 loads are issued together (one by one, with a branch around each, a lone probe
+        // took 88 us, with them 64; all 32 at once take registers from the even placements)
 #pragma unroll
-        for (int yl = 0; yl < 8; ++yl) {
-          int yy = 8 * warp_id + yl - sh.y;
-          if constexpr (CYCLIC) {
-            yy &= (kW - 1);
-          } else if (yy < 0 || yy >= Wu) {
-            continue;
-          }
-          const size_t off = static_cast<size_t>(ti) * (Wu * Wu) + yy * Wu;
+        for (int y4 = 0; y4 < 8; y4 += 4) {
+          using One = typename std::conditional<HALF, unsigned, float2>::type;
+          One buf[16];
 #pragma unroll
-          for (int m = 0; m < 4; ++m) {
-            int xe = 64 * (m >> 1) + 2 * lane_id + (m & 1) - sh.x;
-            if constexpr (CYCLIC) {
-              xe &= (kW - 1);
-            } else if (xe < 0 || xe >= Wu) {
-              continue;
-            }
-            if constexpr (HALF)
-              acc[yl * 4 + m] = cfma(acc[yl * 4 + m], al, __half22float2(static_cast<const __half2*>(Uhc)[off + xe]));
+          for (int yl = 0; yl < 4; ++yl) {
+            int yy = 8 * warp_id + y4 + yl - sh.y;
+            bool oky = true;
+            if constexpr (CYCLIC)
+              yy &= (kW - 1);
             else
-              acc[yl * 4 + m] = cfma(acc[yl * 4 + m], al, Uc[off + xe]);
+              oky = static_cast<unsigned>(yy) < static_cast<unsigned>(Wu);
+            const long long row = static_cast<long long>(ti) * (Wu * Wu) + yy * Wu;
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+              int xe = 64 * (m >> 1) + 2 * lane_id + (m & 1) - sh.x;
+              bool ok = oky;
+              if constexpr (CYCLIC)
+                xe &= (kW - 1);
+              else
+                ok = ok && static_cast<unsigned>(xe) < static_cast<unsigned>(Wu);
+              One v{};
+              if (ok) {
+                if constexpr (HALF)
+                  v = static_cast<const unsigned*>(Uhc)[row + xe];
+                else
+                  v = Uc[row + xe];
+              }
+              buf[yl * 4 + m] = v;
+            }
+          }
+#pragma unroll
+          for (int e = 0; e < 16; ++e) {
+            float2 f;
+            if constexpr (HALF)
+              f = __half22float2(*reinterpret_cast<const __half2*>(&buf[e]));
+            else
+              f = buf[e];
+            acc[y4 * 4 + e] = cfma2(acc[y4 * 4 + e], al4, f);
           }
         }
       }
