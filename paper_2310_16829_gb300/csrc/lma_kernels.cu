@@ -301,8 +301,8 @@ __device__ __forceinline__ void passA_fwd(float2 (&v)[32], const float2* twA) {
 #pragma unroll
   for (int k = 0; k < 32; k += 2) {
     const float4 w = w4[k / 2];
-    if (k > 0) v[k] = cmul(v[k], make_float2(w.x, w.y));
-    v[k + 1] = cmul(v[k + 1], make_float2(w.z, w.w));
+    if (k > 0) v[k] = cmul_xy(v[k], make_float2(w.x, w.y));
+    v[k + 1] = cmul_xy(v[k + 1], make_float2(w.z, w.w));
   }
 }
 
@@ -317,7 +317,7 @@ __device__ __forceinline__ void passB_fwd(float2 (&a)[16], const float2* twB) {
   for (int k1y = 1; k1y < 4; ++k1y) {
     const float2 w = twB[k1y];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) a[k1y * 4 + q] = cmul(a[k1y * 4 + q], w);
+    for (int q = 0; q < 4; ++q) a[k1y * 4 + q] = cmul_xy(a[k1y * 4 + q], w);
   }
 }
 
@@ -2382,6 +2382,174 @@ __device__ __forceinline__ int probe_of(int q, int npx, int npy, int sw) {
   return (r / w) * npx + x0 + (r - (r / w) * w);
 }
 
+// The detection part of the synthesis kernels (passes A, B, C and the readout): the thread's
+// places in the exchange table and its detector bits. A -> B goes through X1, B -> C through X2.
+template <int MODE>
+struct Detect {
+  float2* R0;
+  float* red;
+  const float2 *tA, *tB;
+  float4* x1w;
+  float2 *x1r, *x2b, *x2c;
+  uint32_t dbits[kMaxDet];
+  int kx, k1y, kxs;
+  bool c_live;
+
+  // the twiddle tables, read after a CTA barrier
+  static __device__ __forceinline__ void tables(float2* sm) { load_twiddles(sm + kX1, sm + kX1 + kTwA, threadIdx.x); }
+  __device__ __forceinline__ void places(const SynthArgs& a, float2* sm) {
+    R0 = sm;
+    const float2* const twA = sm + kX1;
+    const float2* const twB = twA + kTwA;
+    red = reinterpret_cast<float*>(sm + kX1 + kTwA + 128);   // [16 warps][kMaxDet]
+    const int T = threadIdx.x;
+    const int ra = T & 3;
+    const int k1lo = T & 15, n2y = T >> 4;
+    kx = c_column(T);
+    k1y = T >> 7;
+    const int k1x = kx & 31, k2x = kx >> 5;
+    tA = twA + ra * 34;
+    tB = twB + n2y * 4;
+    x1w = reinterpret_cast<float4*>(R0 + T * 34);
+    x1r = R0 + (4 * n2y) * 34 + k1lo;
+    x2b = R0 + n2y * 32 + k1lo;
+    x2c = R0 + (k1y * 4 + k2x) * 1024 + k1x;
+    uint32_t any_bits = 0u;
+    kxs = kx < 64 ? kx : kx - 128;
+    if constexpr (MODE == kReadAnnuli) {
+#pragma unroll
+      for (int d = 0; d < kMaxDet; ++d) {
+        dbits[d] = d < a.n_det ? a.det_bits[d * kThreads + kx + 128 * k1y] : 0u;
+        any_bits |= dbits[d];
+      }
+    } else {
+      // labels and the pattern cover in-band pixels only
+      any_bits = kxs * kxs <= a.band_r2 ? 1u : 0u;
+    }
+    // a warp whose columns meet no detector skips pass C
+    c_live = __any_sync(0xffffffffu, any_bits != 0u);
+  }
+
+  // Psi_p of probe p in pass A's layout, v[n1] = Psi_p(y = T / 4, x = 4 n1 + T % 4) -> the readings of
+  // configuration slot cfg. Every thread of the warp has read what it needs of the warp's X1 rows.
+  __device__ __forceinline__ void read(const SynthArgs& a, float2 (&v)[32], const int cfg, const int p) const {
+    const int T = threadIdx.x;
+    // forward 2D DFT of Psi_p (passes A, B, C)
+    passA_fwd(v, tA);
+#pragma unroll
+    for (int k = 0; k < 32; k += 2) x1w[k / 2] = make_float4(v[k].x, v[k].y, v[k + 1].x, v[k + 1].y);
+    __syncthreads();
+    float2 b0[16], b1[16];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        b0[q * 4 + r] = x1r[(128 * q + r) * 34];
+        b1[q * 4 + r] = x1r[(128 * q + r) * 34 + 16];
+      }
+    passB_fwd(b0, tB);
+    passB_fwd(b1, tB);
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        x2b[(q * 4 + r) * 1024] = b0[q * 4 + r];
+        x2b[(q * 4 + r) * 1024 + 16] = b1[q * 4 + r];
+      }
+    __syncthreads();
+    const int warp = T >> 5, lane = T & 31;
+    if constexpr (MODE == kReadAnnuli) {
+      if (c_live) {
+        float2 c[32];
+#pragma unroll
+        for (int j = 0; j < 32; ++j) c[j] = x2c[j * 32];
+        dft32<false>(c);
+        // detector (Sec. 3.1, 2D STEM): sum of |DFT|^2 over the annulus
+#pragma unroll
+        for (int d = 0; d < kMaxDet; ++d) {
+          if (d >= a.n_det) break;
+          float sum = 0.f;
+#pragma unroll
+          for (int j = 0; j < 32; ++j)
+            if ((dbits[d] >> j) & 1u) sum = fmaf(c[j].x, c[j].x, fmaf(c[j].y, c[j].y, sum));
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+          if (lane == 0) red[warp * kMaxDet + d] = sum;
+        }
+      } else if (lane < kMaxDet) {
+        red[warp * kMaxDet + lane] = 0.f;
+      }
+      __syncthreads();
+      if (T < a.n_det) {
+        double tot = 0.0;
+        for (int w = 0; w < kThreads / 32; ++w) tot += static_cast<double>(red[w * kMaxDet + T]);
+        a.acc[(static_cast<size_t>(a.cfg_base + cfg) * a.n_det + T) * a.n_probes + p] = tot * (1.0 / (kW * kW));
+      }
+    } else if constexpr (MODE == kReadLabels) {
+      // 3D STEM (Sec. 3.1): |DFT|^2 into a W x W plane, then each label's pixels summed by
+      // one warp in a fixed order (lane-strided partial sums, then a fixed shuffle tree)
+      float e[32];
+      if (c_live) {
+        float2 c[32];
+#pragma unroll
+        for (int j = 0; j < 32; ++j) c[j] = x2c[j * 32];
+        dft32<false>(c);
+#pragma unroll
+        for (int j = 0; j < 32; ++j) e[j] = fmaf(c[j].x, c[j].x, c[j].y * c[j].y);
+      }
+      __syncthreads();   // every X2 read of R0 is done: R0 becomes the plane
+      float* plane = reinterpret_cast<float*>(R0);
+      if (c_live) {
+#pragma unroll
+        for (int j = 0; j < 32; ++j) plane[(k1y + 4 * j) * kW + kx] = e[j];
+      }
+      __syncthreads();
+      for (int l = warp; l < a.n_det; l += kThreads / 32) {
+        const int s0 = a.lab_start[l], s1 = a.lab_start[l + 1];
+        float sum = 0.f;
+        for (int i = s0 + lane; i < s1; i += 32) sum += plane[a.lab_pix[i]];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if (lane == 0)
+          a.acc[(static_cast<size_t>(a.cfg_base + cfg) * a.n_det + l) * a.n_probes + p] =
+              static_cast<double>(sum) * (1.0 / (kW * kW));
+      }
+    } else {
+      // 4D STEM (Sec. 3.1): the pattern |DFT|^2 / W^2 on |kx| <= pat_a, |ky| <= pat_b, zero
+      // outside the band, one FP32 slot per configuration
+      const int pw = 2 * a.pat_a + 1;
+      float* const out = a.pat + (static_cast<size_t>(cfg) * a.n_probes + p) * static_cast<size_t>(pw * (2 * a.pat_b + 1)) +
+                         a.pat_b * pw + kxs + a.pat_a;
+      const bool col = kxs >= -a.pat_a && kxs <= a.pat_a;
+      if (c_live) {
+        float2 c[32];
+#pragma unroll
+        for (int j = 0; j < 32; ++j) c[j] = x2c[j * 32];
+        dft32<false>(c);
+        if (col) {
+#pragma unroll
+          for (int j = 0; j < 32; ++j) {
+            const int ky = k1y + 4 * j;
+            const int kys = ky < 64 ? ky : ky - 128;
+            if (kys >= -a.pat_b && kys <= a.pat_b)
+              out[kys * pw] = kxs * kxs + kys * kys <= a.band_r2
+                                  ? fmaf(c[j].x, c[j].x, c[j].y * c[j].y) * (1.f / (kW * kW))
+                                  : 0.f;
+          }
+        }
+      } else if (col) {
+#pragma unroll
+        for (int j = 0; j < 32; ++j) {
+          const int ky = k1y + 4 * j;
+          const int kys = ky < 64 ? ky : ky - 128;
+          if (kys >= -a.pat_b && kys <= a.pat_b) out[kys * pw] = 0.f;
+        }
+      }
+    }
+  }
+};
+
 // HALF reads the FP16 store and folds each wave's factor into its coefficient. MODE
 // selects the readout (ReadMode): 2D annuli, labelled pixel sets (3D STEM rings) or the
 // diffraction pattern on a centred crop (4D STEM).
@@ -2390,38 +2558,12 @@ __device__ __forceinline__ int probe_of(int q, int npx, int npy, int sw) {
 template <bool HALF, int MODE, bool CYCLIC, int WS = kW>
 __global__ void __launch_bounds__(kThreads, 1) k_synth_detect(const SynthArgs a) {
   extern __shared__ __align__(16) float2 sm[];
-  float2* R0 = sm;
-  float2* twA = sm + kX1;
-  float2* twB = twA + kTwA;
-  float* red = reinterpret_cast<float*>(twB + 128);   // [16 warps][kMaxDet]
-
-  const int T = threadIdx.x;
-  load_twiddles(twA, twB, T);
-  const int ra = T & 3;
-  const int k1lo = T & 15, n2y = T >> 4;
-  const int kx = c_column(T), k1y = T >> 7, k1x = kx & 31, k2x = kx >> 5;
-  const float2* tA = twA + ra * 34;
-  const float2* tB = twB + n2y * 4;
-  float4* const x1w = reinterpret_cast<float4*>(R0 + T * 34);
-  float2* const x1r = R0 + (4 * n2y) * 34 + k1lo;
-  float2* const x2b = R0 + n2y * 32 + k1lo;
-  float2* const x2c = R0 + (k1y * 4 + k2x) * 1024 + k1x;
-  uint32_t dbits[kMaxDet];
-  uint32_t any_bits = 0u;
-  const int kxs = kx < 64 ? kx : kx - 128;
-  if constexpr (MODE == kReadAnnuli) {
-#pragma unroll
-    for (int d = 0; d < kMaxDet; ++d) {
-      dbits[d] = d < a.n_det ? a.det_bits[d * kThreads + kx + 128 * k1y] : 0u;
-      any_bits |= dbits[d];
-    }
-  } else {
-    // labels and the pattern cover in-band pixels only
-    any_bits = kxs * kxs <= a.band_r2 ? 1u : 0u;
-  }
-  // a warp whose columns meet no detector skips pass C
-  const bool c_live = __any_sync(0xffffffffu, any_bits != 0u);
+  Detect<MODE> det;
+  det.tables(sm);
+  det.places(a, sm);
   __syncthreads();
+  float2* const R0 = sm;
+  const int T = threadIdx.x;
 
   // exit-wave window W (the store's row length); the probe window D is kW. The periodic
   // placement (CYCLIC) has W = D = kW.
@@ -2597,120 +2739,167 @@ __global__ void __launch_bounds__(kThreads, 1) k_synth_detect(const SynthArgs a)
 #pragma unroll
     for (int n1 = 0; n1 < 32; ++n1) v[n1] = tb[(lane_id >> 2) * 132 + 4 * n1 + (lane_id & 3)];
     __syncwarp();      // every lane has read its row before X1 overwrites the warp's rows
-    // forward 2D DFT of Psi_p (passes A, B, C)
-    passA_fwd(v, tA);
+    det.read(a, v, cfg, p);
+  }
+}
+
+// The synthesis of a probe by a cluster of C = 2 or 4 CTAs, for launches too small to give every SM
+// a probe of its own: each CTA sums 128 / C of the pixel rows (warp w of CTA `rank` rows y = R (C w +
+// rank) + r, r < R = 8 / C), then all write their rows into the table of one of them
+// (distributed shared memory, in the layout the transform reads; which one rotates with the
+// probe), which transforms and reads out. The sums are k_synth_detect's: the same products in the
+// same order. 2 (C = 2) or 5 (C = 4) waves' loads are in flight together, against one in
+// k_synth_detect, whose threads hold 32 sums instead of 16 or 8.
+//
+// What bounds it: latency, of the loads' L2 round trips and of the transform. One launch of L = 32,
+// complex64, 36 probes with even (odd) placements: 26 us (29), against 37 (87 with k_synth_detect's
+// odd placements one by one); 72 probes in clusters of two: 33 us (38), against 38 (88).
+namespace split {
+__device__ __forceinline__ void arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ uint32_t remote(const void* p, int rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(p))), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void store4(uint32_t addr, float2 a, float2 b) {
+  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y) : "memory");
+}
+}  // namespace split
+
+// Non-periodic placement; WS as in k_synth_detect.
+template <bool HALF, int MODE, int WS, int C>
+__global__ void __launch_bounds__(kThreads, 1) k_synth_split(const SynthArgs a) {
+  extern __shared__ __align__(16) float2 sm[];
+  constexpr int R = 8 / C, NB = C == 2 ? 2 : 5;   // waves in flight: as many as registers hold
+  using Raw = typename std::conditional<HALF, uint2, float4>::type;
+  Detect<MODE>::tables(sm);   // published by the barriers of the first item
+  float2* const R0 = sm;
+  const int T = threadIdx.x, warp = T >> 5, lane = T & 31;
+  int rank;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+  const int Wu = WS > 0 ? WS : a.W;
+  const int y0 = R * (C * warp + rank);         // the warp's rows
+  const int n_walk = a.probe_list ? a.n_list : a.n_probes;
+  const int n_items = n_walk * a.n_cfg;
+  split::arrive();
+  for (int item = blockIdx.x / C; item < n_items; item += gridDim.x / C) {
+    const int cfg = item / n_walk, q = item - cfg * n_walk;
+    const int p = a.probe_list ? a.probe_list[q] : probe_of(q, a.npx, a.npy, a.strip);
+    const size_t t0 = static_cast<size_t>(a.probe_list ? q : p) * a.L;
+    const float2* const Uc = a.U ? a.U + cfg * a.u_slot : nullptr;
+    const __half2* const Uhc = a.Uh ? static_cast<const __half2*>(a.Uh) + cfg * a.u_slot : nullptr;
+    const float* const Usc = a.Uscale ? a.Uscale + static_cast<size_t>(cfg) * a.n_translates : nullptr;
+    float2 acc[R][4];
 #pragma unroll
-    for (int k = 0; k < 32; k += 2) x1w[k / 2] = make_float4(v[k].x, v[k].y, v[k + 1].x, v[k + 1].y);
-    __syncthreads();
-    float2 b0[16], b1[16];
+    for (int r = 0; r < R; ++r)
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
+      for (int m = 0; m < 4; ++m) acc[r][m] = make_float2(0.f, 0.f);
+    // lane l holds columns 64 kk + 2 l + e of the rows, as in k_synth_detect
+#pragma unroll 1
+    for (int j0 = 0; j0 < a.L; j0 += NB) {
+      Raw buf[NB][R][2];
+      float2 al[NB];
 #pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        b0[q * 4 + r] = x1r[(128 * q + r) * 34];
-        b1[q * 4 + r] = x1r[(128 * q + r) * 34 + 16];
-      }
-    passB_fwd(b0, tB);
-    passB_fwd(b1, tB);
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        x2b[(q * 4 + r) * 1024] = b0[q * 4 + r];
-        x2b[(q * 4 + r) * 1024 + 16] = b1[q * 4 + r];
-      }
-    __syncthreads();
-    const int warp = T >> 5, lane = T & 31;
-    if constexpr (MODE == kReadAnnuli) {
-      if (c_live) {
-        float2 c[32];
-#pragma unroll
-        for (int j = 0; j < 32; ++j) c[j] = x2c[j * 32];
-        dft32<false>(c);
-        // detector (Sec. 3.1, 2D STEM): sum of |DFT|^2 over the annulus
-#pragma unroll
-        for (int d = 0; d < kMaxDet; ++d) {
-          if (d >= a.n_det) break;
-          float sum = 0.f;
-#pragma unroll
-          for (int j = 0; j < 32; ++j)
-            if ((dbits[d] >> j) & 1u) sum = fmaf(c[j].x, c[j].x, fmaf(c[j].y, c[j].y, sum));
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-          if (lane == 0) red[warp * kMaxDet + d] = sum;
+      for (int b = 0; b < NB; ++b) {
+        const bool on = j0 + b < a.L;
+        const size_t e = t0 + min(j0 + b, a.L - 1);
+        const int2 sh = a.shift[e];
+        const int ti = a.tidx[e];
+        al[b] = a.alpha[e];
+        if constexpr (HALF) {
+          const float f = Usc[ti];
+          al[b].x *= f;
+          al[b].y *= f;
         }
-      } else if (lane < kMaxDet) {
-        red[warp * kMaxDet + lane] = 0.f;
-      }
-      __syncthreads();
-      if (T < a.n_det) {
-        double tot = 0.0;
-        for (int w = 0; w < kThreads / 32; ++w) tot += static_cast<double>(red[w * kMaxDet + T]);
-        a.acc[(static_cast<size_t>(a.cfg_base + cfg) * a.n_det + T) * a.n_probes + p] = tot * (1.0 / (kW * kW));
-      }
-    } else if constexpr (MODE == kReadLabels) {
-      // 3D STEM (Sec. 3.1): |DFT|^2 into a W x W plane, then each label's pixels summed by
-      // one warp in a fixed order (lane-strided partial sums, then a fixed shuffle tree)
-      float e[32];
-      if (c_live) {
-        float2 c[32];
+        const int yw = y0 - sh.y, xw = 2 * lane - sh.x;
+        const long long base = static_cast<long long>(ti) * (Wu * Wu) + yw * Wu + xw;
+        const bool pair = (sh.x & 1) == 0;   // column pairs stay aligned and unbroken
 #pragma unroll
-        for (int j = 0; j < 32; ++j) c[j] = x2c[j * 32];
-        dft32<false>(c);
+        for (int r = 0; r < R; ++r) {
+          const bool oky = on && static_cast<unsigned>(yw + r) < static_cast<unsigned>(Wu);
 #pragma unroll
-        for (int j = 0; j < 32; ++j) e[j] = fmaf(c[j].x, c[j].x, c[j].y * c[j].y);
-      }
-      __syncthreads();   // every X2 read of R0 is done: R0 becomes the plane
-      float* plane = reinterpret_cast<float*>(R0);
-      if (c_live) {
-#pragma unroll
-        for (int j = 0; j < 32; ++j) plane[(k1y + 4 * j) * kW + kx] = e[j];
-      }
-      __syncthreads();
-      for (int l = warp; l < a.n_det; l += kThreads / 32) {
-        const int s0 = a.lab_start[l], s1 = a.lab_start[l + 1];
-        float sum = 0.f;
-        for (int i = s0 + lane; i < s1; i += 32) sum += plane[a.lab_pix[i]];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-        if (lane == 0)
-          a.acc[(static_cast<size_t>(a.cfg_base + cfg) * a.n_det + l) * a.n_probes + p] =
-              static_cast<double>(sum) * (1.0 / (kW * kW));
-      }
-    } else {
-      // 4D STEM (Sec. 3.1): the pattern |DFT|^2 / W^2 on |kx| <= pat_a, |ky| <= pat_b, zero
-      // outside the band, one FP32 slot per configuration
-      const int pw = 2 * a.pat_a + 1;
-      float* const out = a.pat + (static_cast<size_t>(cfg) * a.n_probes + p) * static_cast<size_t>(pw * (2 * a.pat_b + 1)) +
-                         a.pat_b * pw + kxs + a.pat_a;
-      const bool col = kxs >= -a.pat_a && kxs <= a.pat_a;
-      if (c_live) {
-        float2 c[32];
-#pragma unroll
-        for (int j = 0; j < 32; ++j) c[j] = x2c[j * 32];
-        dft32<false>(c);
-        if (col) {
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            const int ky = k1y + 4 * j;
-            const int kys = ky < 64 ? ky : ky - 128;
-            if (kys >= -a.pat_b && kys <= a.pat_b)
-              out[kys * pw] = kxs * kxs + kys * kys <= a.band_r2
-                                  ? fmaf(c[j].x, c[j].x, c[j].y * c[j].y) * (1.f / (kW * kW))
-                                  : 0.f;
+          for (int kk = 0; kk < 2; ++kk) {
+            // only elements inside the window are read; the others count as zero
+            const bool k0 = oky && static_cast<unsigned>(xw + 64 * kk) < static_cast<unsigned>(Wu);
+            const bool k1 = oky && static_cast<unsigned>(xw + 64 * kk + 1) < static_cast<unsigned>(Wu);
+            const long long o = base + (r * Wu + 64 * kk);
+            Raw v{};
+            if constexpr (HALF) {
+              if (pair) {
+                if (k0) v = *reinterpret_cast<const uint2*>(Uhc + o);
+              } else {
+                if (k0) v.x = *reinterpret_cast<const unsigned*>(Uhc + o);
+                if (k1) v.y = *reinterpret_cast<const unsigned*>(Uhc + o + 1);
+              }
+            } else {
+              if (pair) {
+                if (k0) v = *reinterpret_cast<const float4*>(Uc + o);
+              } else {
+                if (k0) {
+                  const float2 f = Uc[o];
+                  v.x = f.x;
+                  v.y = f.y;
+                }
+                if (k1) {
+                  const float2 f = Uc[o + 1];
+                  v.z = f.x;
+                  v.w = f.y;
+                }
+              }
+            }
+            buf[b][r][kk] = v;
           }
         }
-      } else if (col) {
+      }
 #pragma unroll
-        for (int j = 0; j < 32; ++j) {
-          const int ky = k1y + 4 * j;
-          const int kys = ky < 64 ? ky : ky - 128;
-          if (kys >= -a.pat_b && kys <= a.pat_b) out[kys * pw] = 0.f;
-        }
+      for (int b = 0; b < NB; ++b) {
+        if (j0 + b >= a.L) break;
+        const float4 al4 = make_float4(al[b].x, al[b].x, -al[b].y, al[b].y);   // cfma2's form of the coefficient
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+          for (int kk = 0; kk < 2; ++kk) {
+            float2 f0, f1;
+            if constexpr (HALF) {
+              f0 = __half22float2(*reinterpret_cast<const __half2*>(&buf[b][r][kk].x));
+              f1 = __half22float2(*reinterpret_cast<const __half2*>(&buf[b][r][kk].y));
+            } else {
+              f0 = make_float2(buf[b][r][kk].x, buf[b][r][kk].y);
+              f1 = make_float2(buf[b][r][kk].z, buf[b][r][kk].w);
+            }
+            acc[r][2 * kk] = cfma2(acc[r][2 * kk], al4, f0);
+            acc[r][2 * kk + 1] = cfma2(acc[r][2 * kk + 1], al4, f1);
+          }
       }
     }
+    // row y = 8 w + yl goes to w * 1088 + yl * 132 of the reader's table (the reading warp's own X1 rows)
+    split::wait();                               // every CTA of the cluster is past its last transform
+    const uint32_t dst = split::remote(R0, item % C);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int y = y0 + r;
+#pragma unroll
+      for (int kk = 0; kk < 2; ++kk)
+        split::store4(dst + 8u * static_cast<uint32_t>((y >> 3) * (32 * 34) + (y & 7) * 132 + 64 * kk + 2 * lane), acc[r][2 * kk],
+                      acc[r][2 * kk + 1]);
+    }
+    split::arrive();
+    split::wait();
+    if (rank == item % C) {
+      const float2* const tb = R0 + warp * (32 * 34);
+      float2 v[32];
+#pragma unroll
+      for (int n1 = 0; n1 < 32; ++n1) v[n1] = tb[(lane >> 2) * 132 + 4 * n1 + (lane & 3)];
+      __syncwarp();      // every lane has read its row before X1 overwrites the warp's rows
+      Detect<MODE> det;
+      det.places(a, sm);
+      det.read(a, v, cfg, p);
+    }
+    __syncwarp();
+    split::arrive();
   }
+  split::wait();
 }
 
 // Step a4 for a group of neighbouring probes. The group's frame is the union of its probe
@@ -3142,6 +3331,9 @@ size_t slice_gen_scratch_bytes(int W) {
 }
 size_t slice_rs_smem_bytes() { return static_cast<size_t>(kW * kW + 32 * 32) * sizeof(float2); }
 
+using SynthKernel = void (*)(const SynthArgs);
+template <int C>
+static SynthKernel synth_split_kernel(bool half, int mode, bool other_w);
 cudaError_t init_device_constants() {
   float2 w[128];
   const double pi = 3.14159265358979323846;
@@ -3246,6 +3438,10 @@ cudaError_t init_device_constants() {
                  k_synth_detect<false, kReadAnnuli, false, 0>, k_synth_detect<false, kReadLabels, false, 0>,
                  k_synth_detect<false, kReadPattern, false, 0>})
     if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, sy)) != cudaSuccess) return e;
+  for (int m : {kReadAnnuli, kReadLabels, kReadPattern})
+    for (int v = 0; v < 3; ++v)
+      for (SynthKernel f : {synth_split_kernel<2>(v == 1, m, v == 2), synth_split_kernel<4>(v == 1, m, v == 2)})
+        if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, sy)) != cudaSuccess) return e;
   for (auto f : {k_synth_group<false>, k_synth_group<true>})
     if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   static_cast<int>(synth_group_smem_bytes()))) != cudaSuccess)
@@ -3376,6 +3572,40 @@ cudaError_t launch_slice_rs(const SliceLaunch& a, const float2* q, int K1, int K
   return cudaGetLastError();
 }
 
+template <int C>
+static SynthKernel synth_split_kernel(bool half, int mode, bool other_w) {
+  static const SynthKernel table[3][3] = {
+      {k_synth_split<false, kReadAnnuli, kW, C>, k_synth_split<false, kReadLabels, kW, C>, k_synth_split<false, kReadPattern, kW, C>},
+      {k_synth_split<true, kReadAnnuli, kW, C>, k_synth_split<true, kReadLabels, kW, C>, k_synth_split<true, kReadPattern, kW, C>},
+      {k_synth_split<false, kReadAnnuli, 0, C>, k_synth_split<false, kReadLabels, 0, C>, k_synth_split<false, kReadPattern, 0, C>}};
+  return table[other_w ? 2 : (half ? 1 : 0)][mode == kReadAnnuli ? 0 : (mode == kReadLabels ? 1 : 2)];
+}
+static void cluster_config(cudaLaunchConfig_t& cfg, cudaLaunchAttribute& at, int ctas, int clusters, cudaStream_t s) {
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = static_cast<unsigned>(ctas);
+  at.val.clusterDim.y = 1;
+  at.val.clusterDim.z = 1;
+  cfg.gridDim = dim3(static_cast<unsigned>(ctas) * static_cast<unsigned>(clusters));
+  cfg.blockDim = dim3(kThreads);
+  cfg.dynamicSmemBytes = synth_smem_bytes();
+  cfg.stream = s;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+}
+// clusters of C CTAs that the device holds at once (one CTA per SM; a GPC's SMs need not be a
+// multiple of C)
+template <int C>
+static int split_clusters() {
+  static const int n = [] {
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at{};
+    cluster_config(cfg, at, C, sm_count(), nullptr);
+    int k = 0;
+    return cudaOccupancyMaxActiveClusters(&k, k_synth_split<false, kReadAnnuli, kW, C>, &cfg) == cudaSuccess ? k : 0;
+  }();
+  return n;
+}
+
 cudaError_t launch_synth(const SynthArgs& a, bool half, int mode, int grid_mode, cudaStream_t s) {
   const int n_walk = a.probe_list ? a.n_list : a.n_probes;
   if (n_walk <= 0) return cudaSuccess;
@@ -3387,6 +3617,18 @@ cudaError_t launch_synth(const SynthArgs& a, bool half, int mode, int grid_mode,
   const bool persistent = grid_mode == kSynthGridPersistent || (grid_mode == kSynthGridAuto && !half);
   const int grid = persistent ? (n_items < sm_count() ? n_items : sm_count()) : n_items;
   const size_t sm = synth_smem_bytes();
+  // several CTAs per probe while the clusters fit the device at once. In a second round the
+  // clusters of four lose to one CTA per probe (72 probes: 47 us against 38), so pairs take over,
+  // and from half the SMs on k_synth_detect (81 probes: 38 us).
+  if (grid_mode == kSynthGridAuto && !a.cyclic && n_items <= split_clusters<2>()) {
+    if ((mode != kReadAnnuli && mode != kReadLabels && mode != kReadPattern) || (a.W != kW && (half || a.W < 32 || a.W > 256)))
+      return cudaErrorInvalidValue;
+    const bool four = n_items <= split_clusters<4>();
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at{};
+    cluster_config(cfg, at, four ? 4 : 2, n_items, s);
+    return cudaLaunchKernelEx(&cfg, four ? synth_split_kernel<4>(half, mode, a.W != kW) : synth_split_kernel<2>(half, mode, a.W != kW), a);
+  }
   // periodic probe windows (the window is the whole cell) wrap; others are zero outside
   using K = void (*)(const SynthArgs);
   static const K table[2][3][2] = {
