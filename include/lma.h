@@ -320,7 +320,8 @@ lma_status lma_image_realspace(lma_ctx* ctx, lma_specimen* spec, lma_basis* basi
 
 /* Self-test of the bounded device waits. The tensor-core slice kernel (LMA_PREC_MIXED) and
  * the W = 256 slice kernel wait on shared-memory mbarriers for the MMAs and bulk copies they
- * issue, each wait one polling lane per warp with at most 2000 suspended tries of up to 1 ms;
+ * issue, each wait a few tries by every lane of a warp, then one polling lane with at most 2000
+ * suspended tries of up to 1 ms;
  * a wait that gives up sets the launch's status word, the kernel returns, and the next call
  * that reads results returns LMA_ERR_TIMEOUT. This call runs that wait on an mbarrier phase
  * that nothing completes, in one warp (which = 0, as in the tensor-core kernel's per-tile

@@ -800,6 +800,7 @@ __device__ __forceinline__ uint32_t try_wait(uint32_t mbar, uint32_t phase) {
 // (woken when it completes), instead of spinning on the shared-memory pipe
 constexpr uint32_t kSuspendNs = 1000000;
 constexpr int kSuspendLimit = 2000;          // at least 2 s in all before giving up
+constexpr int kWarpTries = 8;
 __device__ __forceinline__ uint32_t try_wait_sleep(uint32_t mbar, uint32_t phase) {
   uint32_t done;
   asm volatile(
@@ -816,10 +817,13 @@ __device__ __forceinline__ bool wait_phase(uint32_t mbar, uint32_t phase) {
   for (int it = 0; it < kSuspendLimit && !done; ++it) done = try_wait_sleep(mbar, phase);
   return done != 0;
 }
-// the same for a whole warp: lane 0 polls, then every lane observes the completed phase
+// the same for a whole warp: a few tries by every lane (the wait of a pass is short), then lane 0
+// polls and every lane observes the completed phase
 // itself (one try_wait each, for the memory ordering), so 31 lanes do not spin on the
 // shared-memory pipe; warp-uniform result
 __device__ __forceinline__ bool wait_phase_warp(uint32_t mbar, uint32_t phase) {
+  for (int it = 0; it < kWarpTries; ++it)
+    if (__all_sync(0xffffffffu, try_wait(mbar, phase) != 0)) return true;
   uint32_t done = 0;
   if ((threadIdx.x & 31) == 0) done = wait_phase(mbar, phase) ? 1u : 0u;
   done = __shfl_sync(0xffffffffu, done, 0);
@@ -830,50 +834,52 @@ __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::be
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
-// the 64 FP32 columns of this thread's TMEM lane from column c: y[k] = (col k, col 32 + k)
-__device__ __forceinline__ void load_row(uint32_t taddr, float2 (&y)[32]) {
-  uint32_t r[64];
+// half h of the complex values of this thread's TMEM row: y[k] = value 16 h + k = columns 2 (16 h + k)
+// and the next, so that the loaded registers are the values' pairs. Halves keep 32 registers
+// live instead of 64 between the accumulators and their next place.
+__device__ __forceinline__ void load_half(uint32_t taddr, int h, float2* y) {
+  uint32_t r[32];
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x64.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32,%33,%34,%35,%36,%37,%38,%39,"
-      "%40,%41,%42,%43,%44,%45,%46,%47,%48,%49,%50,%51,%52,%53,%54,%55,%56,%57,%58,%59,%60,%61,%62,%63}, [%64];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31]),
-        "=r"(r[32]), "=r"(r[33]), "=r"(r[34]), "=r"(r[35]), "=r"(r[36]), "=r"(r[37]), "=r"(r[38]), "=r"(r[39]),
-        "=r"(r[40]), "=r"(r[41]), "=r"(r[42]), "=r"(r[43]), "=r"(r[44]), "=r"(r[45]), "=r"(r[46]), "=r"(r[47]),
-        "=r"(r[48]), "=r"(r[49]), "=r"(r[50]), "=r"(r[51]), "=r"(r[52]), "=r"(r[53]), "=r"(r[54]), "=r"(r[55]),
-        "=r"(r[56]), "=r"(r[57]), "=r"(r[58]), "=r"(r[59]), "=r"(r[60]), "=r"(r[61]), "=r"(r[62]), "=r"(r[63])
-      : "r"(taddr)
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr + 32 * h)
       : "memory");
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-  for (int k = 0; k < 32; ++k) y[k] = make_float2(__uint_as_float(r[k]), __uint_as_float(r[32 + k]));
+  for (int k = 0; k < 16; ++k) y[k] = make_float2(__uint_as_float(r[2 * k]), __uint_as_float(r[2 * k + 1]));
+}
+__device__ __forceinline__ void load_row(uint32_t taddr, float2 (&y)[32]) {
+  load_half(taddr, 0, y);
+  load_half(taddr, 1, y + 16);
 }
 
-// Row `row` of a tile's A operand from x: K index k < 32 holds Re x[k], k >= 32 Im x[k - 32];
-// high parts to `hi`, low parts to `lo` (16-byte stores: a quarter-warp's 8 rows fill 128
-// contiguous bytes)
-__device__ __forceinline__ void store_row(unsigned char* hi, unsigned char* lo, const float2 (&x)[32], int row) {
-  const uint32_t base = op_offset(row, 0);
+// Half h (values 16 h .. 16 h + 15) of row `row` of a tile's A operand: K index k < 32 holds Re
+// x[k], k >= 32 Im x[k - 32]; high parts to `hi`, low parts to `lo` (16-byte stores: a
+// quarter-warp's 8 rows fill 128 contiguous bytes)
+__device__ __forceinline__ void store_half(unsigned char* hi, unsigned char* lo, const float2* x, int row, int hf) {
+  const uint32_t base = op_offset(row, 0) + 256 * hf;
 #pragma unroll
-  for (int kb = 0; kb < 8; ++kb) {
+  for (int kb = 0; kb < 4; ++kb) {
     uint32_t h[4], l[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const int n = (kb & 3) * 8 + 2 * q;
-      const float a = kb < 4 ? x[n].x : x[n].y;
-      const float b = kb < 4 ? x[n + 1].x : x[n + 1].y;
+      const int n = (kb & 1) * 8 + 2 * q;
+      const float a = kb < 2 ? x[n].x : x[n].y;
+      const float b = kb < 2 ? x[n + 1].x : x[n + 1].y;
       const __half2 hh = __floats2half2_rn(a, b);
-      const float2 hf = __half22float2(hh);
-      const __half2 ll = __floats2half2_rn(a - hf.x, b - hf.y);
+      const float2 hf2 = __half22float2(hh);
+      const __half2 ll = __floats2half2_rn(a - hf2.x, b - hf2.y);
       h[q] = *reinterpret_cast<const uint32_t*>(&hh);
       l[q] = *reinterpret_cast<const uint32_t*>(&ll);
     }
-    *reinterpret_cast<uint4*>(hi + base + kb * 128) = make_uint4(h[0], h[1], h[2], h[3]);
-    *reinterpret_cast<uint4*>(lo + base + kb * 128) = make_uint4(l[0], l[1], l[2], l[3]);
+    const uint32_t at = base + (kb & 1) * 128 + (kb >> 1) * 512;
+    *reinterpret_cast<uint4*>(hi + at) = make_uint4(h[0], h[1], h[2], h[3]);
+    *reinterpret_cast<uint4*>(lo + at) = make_uint4(l[0], l[1], l[2], l[3]);
   }
+}
+__device__ __forceinline__ void store_row(unsigned char* hi, unsigned char* lo, const float2 (&x)[32], int row) {
+  store_half(hi, lo, x, row, 0);
+  store_half(hi, lo, x + 16, row, 1);
 }
 
 // the MMAs of one pass over the four tiles: forward D = A B (N = 64), inverse by sub-blocks
@@ -922,6 +928,12 @@ constexpr int kSliceTcSmemBytes = kXRows * 8 + 4 * tc::kBBytes + 64 * 16 + 128 *
 // rows are the same in passes A and B (as in k_slice: X1 and X4 need __syncwarp). CTA
 // barriers remain where data cross tiles: X2 and X3, the reads of X2 before pass C's operands
 // overwrite the table, and the X3 writes after every tile's inverse pass C.
+//
+// What bounds it: latency between the passes' steps (split, store, products, read back) with one
+// translate per SM, and registers: accumulators are read back in halves and pass B runs one half of
+// k1 at a time, which took spills and stalls out (16384 translates x 20 slices: 41.8 -> 36.2 ms;
+// halves of the read-back and complex values in neighbouring columns 39.4, a few plain tries
+// before a wait suspends 38.4, halves of pass B 36.2).
 template <bool EVEN, bool PRUNE>
 __global__ void __launch_bounds__(kThreads, 1) k_slice_tc(const SliceLaunch a, int* status) {
   extern __shared__ __align__(1024) unsigned char smraw[];
@@ -1047,30 +1059,38 @@ __global__ void __launch_bounds__(kThreads, 1) k_slice_tc(const SliceLaunch a, i
       tc::tile_sync(tile);
       tc::store_row(aHi, aLo, v, arow);
       round(std::false_type{});
-      tc::load_row(t_row, v);
       // X1: this row's pass-A outputs, in the tile's own rows (its MMAs are complete)
       float4* const xa4 = reinterpret_cast<float4*>(xa);
 #pragma unroll
-      for (int k = 0; k < 32; k += 2) xa4[k / 2] = make_float4(v[k].x, v[k].y, v[k + 1].x, v[k + 1].y);
+      for (int h = 0; h < 2; ++h) {
+        float2 y[16];
+        tc::load_half(t_row, h, y);
+#pragma unroll
+        for (int k = 0; k < 16; k += 2) xa4[8 * h + k / 2] = make_float4(y[k].x, y[k].y, y[k + 1].x, y[k + 1].y);
+      }
       __syncwarp();
-      float2 b0[16], b1[16];
+      // pass B one half (k1 < 16, k1 >= 16) at a time: 32 registers live beside the kernel's own
+      {
+        float2 b[16];
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
+        for (int e = 0; e < 16; ++e) b[e] = xb[e * kXP];
+        passB_fwd_tw<false, PRUNE>(b, tB, twr[k1lo], twr[32 + k1lo]);
+        static_for<0, 4>([&](auto qq) {
+          constexpr int q = decltype(qq)::value;
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          b0[q * 4 + r] = xb[(4 * q + r) * kXP];
-          b1[q * 4 + r] = xb[(4 * q + r) * kXP + 16];
-        }
-      passB_fwd_tw<false, PRUNE>(b0, tB, twr[k1lo], twr[32 + k1lo]);
-      passB_fwd_tw<true, PRUNE>(b1, tB, twr[16 + k1lo], twr[48 + k1lo]);
-      static_for<0, 4>([&](auto qq) {
-        constexpr int q = decltype(qq)::value;
+          for (int r = 0; r < 4; ++r)
+            if constexpr (q != masked_k2x<false, PRUNE>()) xb[(4 * x2_slot(q) + r) * kXP] = b[r * 4 + q];
+        });
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          if constexpr (q != masked_k2x<false, PRUNE>()) xb[(4 * x2_slot(q) + r) * kXP] = b0[r * 4 + q];
-          if constexpr (q != masked_k2x<true, PRUNE>()) xb[(4 * x2_slot(q) + r) * kXP + 16] = b1[r * 4 + q];
-        }
-      });
+        for (int e = 0; e < 16; ++e) b[e] = xb[e * kXP + 16];
+        passB_fwd_tw<true, PRUNE>(b, tB, twr[16 + k1lo], twr[48 + k1lo]);
+        static_for<0, 4>([&](auto qq) {
+          constexpr int q = decltype(qq)::value;
+#pragma unroll
+          for (int r = 0; r < 4; ++r)
+            if constexpr (q != masked_k2x<true, PRUNE>()) xb[(4 * x2_slot(q) + r) * kXP + 16] = b[r * 4 + q];
+        });
+      }
       if (__syncthreads_or(bad)) goto abort;
       // pass C forward: every row of X2 is read before the operands overwrite the table
       float2 c[32];
@@ -1082,44 +1102,60 @@ __global__ void __launch_bounds__(kThreads, 1) k_slice_tc(const SliceLaunch a, i
       if (c_live) tc::store_row(aHi, aLo, c, arow);
       round(std::false_type{});
       if (c_live) {
-        tc::load_row(t_row, c);
-        // propagation (Sec. 3.2): exp(-i pi lambda eps |k|^2), bandlimit, 2^-7
+        // propagation (Sec. 3.2): exp(-i pi lambda eps |k|^2), bandlimit, 2^-7; the tile's MMAs have
+        // read its operands
 #pragma unroll
-        for (int j = 0; j < 32; ++j) c[j] = cmul(c[j], j < 16 ? pp[4 * j] : pm[-4 * j]);
-        tc::store_row(aHi, aLo, c, arow);   // the tile's MMAs have read its operands
+        for (int h = 0; h < 2; ++h) {
+          float2 y[16];
+          tc::load_half(t_row, h, y);
+#pragma unroll
+          for (int k = 0; k < 16; ++k) {
+            const int j = 16 * h + k;
+            y[k] = PRUNE && in_gap(j) ? make_float2(0.f, 0.f) : cmul(y[k], j < 16 ? pp[4 * j] : pm[-4 * j]);
+          }
+          tc::store_half(aHi, aLo, y, arow, h);
+        }
       }
       round(std::true_type{});
-      if (c_live) tc::load_row(t_row, c);
       // X3 goes to every tile's rows: every tile's inverse products must be complete
 #pragma unroll 1
       for (int u = 0; u < 4; ++u)
         if (u != tile) bad |= !tc::wait_phase_warp(tc::smem_u32(mbar + u), phase ^ 1);
       if (c_live) {
 #pragma unroll
-        for (int j = 0; j < 32; ++j) xc[j * 16 * kXP] = c[j];
+        for (int h = 0; h < 2; ++h) {
+          float2 y[16];
+          tc::load_half(t_row, h, y);
+#pragma unroll
+          for (int k = 0; k < 16; ++k) xc[(16 * h + k) * 16 * kXP] = y[k];
+        }
       } else if (!PRUNE || (k2x == 1 && k1x < 16)) {   // the masked columns that pass B reads
 #pragma unroll
         for (int j = 0; j < 32; ++j) xc[j * 16 * kXP] = make_float2(0.f, 0.f);
       }
       tc::fence_before();
       if (__syncthreads_or(bad)) goto abort;
-      static_for<0, 4>([&](auto qq) {
-        constexpr int q = decltype(qq)::value;
+      {
+        float2 b[16];
+        static_for<0, 4>([&](auto qq) {
+          constexpr int q = decltype(qq)::value;
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          if constexpr (q != masked_k2x<false, PRUNE>()) b0[r * 4 + q] = xb[(4 * x2_slot(q) + r) * kXP];
-          if constexpr (q != masked_k2x<true, PRUNE>()) b1[r * 4 + q] = xb[(4 * x2_slot(q) + r) * kXP + 16];
-        }
-      });
-      passB_inv_tw<false, PRUNE>(b0, tB, twr[k1lo], twr[32 + k1lo]);
-      passB_inv_tw<true, PRUNE>(b1, tB, twr[16 + k1lo], twr[48 + k1lo]);
+          for (int r = 0; r < 4; ++r)
+            if constexpr (q != masked_k2x<false, PRUNE>()) b[r * 4 + q] = xb[(4 * x2_slot(q) + r) * kXP];
+        });
+        passB_inv_tw<false, PRUNE>(b, tB, twr[k1lo], twr[32 + k1lo]);
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
+        for (int e = 0; e < 16; ++e) xb[e * kXP] = b[e];
+        static_for<0, 4>([&](auto qq) {
+          constexpr int q = decltype(qq)::value;
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          xb[(4 * q + r) * kXP] = b0[q * 4 + r];
-          xb[(4 * q + r) * kXP + 16] = b1[q * 4 + r];
-        }
+          for (int r = 0; r < 4; ++r)
+            if constexpr (q != masked_k2x<true, PRUNE>()) b[r * 4 + q] = xb[(4 * x2_slot(q) + r) * kXP + 16];
+        });
+        passB_inv_tw<true, PRUNE>(b, tB, twr[16 + k1lo], twr[48 + k1lo]);
+#pragma unroll
+        for (int e = 0; e < 16; ++e) xb[e * kXP + 16] = b[e];
+      }
       __syncwarp();
       {
         const float4* const xa4r = reinterpret_cast<const float4*>(xa);
@@ -3382,17 +3418,17 @@ cudaError_t init_device_constants() {
       if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, ss)) != cudaSuccess) return e;
   }
   {
-    // B^T[n][k] of the 32-point DFT in real form (n: output column of [Re y | Im y], k: input
-    // of [Re x | Im x]; F[k][n] = exp(-2 pi i k n / 32)), split into FP16 high and low parts;
+    // B^T[n][k] of the 32-point DFT in real form (n: output column, Re y[0], Im y[0], Re y[1], ..; k:
+    // input of [Re x | Im x]; F[k][n] = exp(-2 pi i k n / 32)), split into FP16 high and low parts;
     // then the same for conj F (the inverse): the off-diagonal blocks change sign
     std::vector<unsigned char> bt(4 * tc::kBBytes, 0);
     for (int inv = 0; inv < 2; ++inv)
       for (int n = 0; n < 64; ++n)
         for (int k = 0; k < 64; ++k) {
-          const int kk = k & 31, nn = n & 31;
+          const int kk = k & 31, nn = n >> 1;
           const double th = 2.0 * pi * ((kk * nn) & 31) / 32.0;
           const double fr = cos(th), fi = inv ? sin(th) : -sin(th);
-          const double val = n < 32 ? (k < 32 ? fr : -fi) : (k < 32 ? fi : fr);
+          const double val = (n & 1) == 0 ? (k < 32 ? fr : -fi) : (k < 32 ? fi : fr);
           const __half hi = __float2half_rn(static_cast<float>(val));
           const __half lo = __float2half_rn(static_cast<float>(val - static_cast<double>(__half2float(hi))));
           const size_t base = static_cast<size_t>(inv) * 2 * tc::kBBytes;
