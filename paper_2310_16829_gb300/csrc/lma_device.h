@@ -104,6 +104,9 @@ struct SynthArgs {
   const uint32_t* det_bits;    // [n_det][kThreads] detector bits in C layout
   int n_det;                   // annuli: detectors; labels: labels (outputs per probe)
   double* acc;                 // [configuration][n_det][n_probes] readings (assigned)
+  // launch_synth_variants: variant v (of kSynthVariants) has its coefficients at alpha + v
+  // alpha_stride and its readings at acc + v acc_stride
+  size_t alpha_stride, acc_stride;
   // kReadLabels: pixel lists of the labels (3D STEM rings), CSR over pixel ky * W + kx
   const int32_t* lab_start;    // [n_det + 1]
   const int32_t* lab_pix;      // ascending pixel indices of each label
@@ -153,6 +156,11 @@ cudaError_t launch_selftest_wait(int which, int* status, cudaStream_t s);
 // FP16 store), one CTA per item, or persistent (one CTA per SM); every grid gives the same bits
 constexpr int kSynthGridAuto = 0, kSynthGridPerItem = 1, kSynthGridPersistent = 2;
 cudaError_t launch_synth(const SynthArgs& a, bool half, int mode, int grid_mode, cudaStream_t s);
+// annular readings of kSynthVariants coefficient sets over the same waves in one launch (the bits of
+// one launch_synth each); synth_variants_fit: whether the launch admits it
+constexpr int kSynthVariants = 4;
+bool synth_variants_fit(const SynthArgs& a, bool half);
+cudaError_t launch_synth_variants(const SynthArgs& a, bool half, cudaStream_t s);
 
 // Step a4 for groups of neighbouring probes (probe_list null, non-periodic placement): each
 // CTA takes gx x gy probes of the region, forms the union of their (translate, placement)

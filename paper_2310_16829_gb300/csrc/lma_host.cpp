@@ -2782,6 +2782,16 @@ lma_status lma_image_coherent(lma_ctx* ctx, lma_specimen* sp, lma_basis* b, cons
       a.n_det = n_det;
       a.acc = static_cast<double*>(b->d_acc.p) + static_cast<size_t>(v) * nph * nout;
       a.band_r2 = b->r2max;
+      // four variants in one launch where the gather serves them (no autotuning, no forced grouped form)
+      if (n_var - v >= lma_dev::kSynthVariants && !ctx->autotune && ctx->synth_mode != LMA_SYNTH_GROUPED &&
+          lma_dev::synth_variants_fit(a, half)) {
+        a.alpha_stride = static_cast<size_t>(np) * L;
+        a.acc_stride = static_cast<size_t>(nph) * nout;
+        CUDA_TRY(ctx, counted(ctx, K_SYNTH, np * nb * lma_dev::kSynthVariants, st,
+                              [&] { return lma_dev::launch_synth_variants(a, half, st); }));
+        v += lma_dev::kSynthVariants - 1;
+        continue;
+      }
       { const lma_status ss_ = synth_launch(ctx, a, half, lma_dev::kReadAnnuli, np * nb, region_geom(b), st); if (ss_ != LMA_OK) return ss_; }
     }
   }

@@ -2479,8 +2479,9 @@ struct Detect {
   }
 
   // Psi_p of probe p in pass A's layout, v[n1] = Psi_p(y = T / 4, x = 4 n1 + T % 4) -> the readings of
-  // configuration slot cfg. Every thread of the warp has read what it needs of the warp's X1 rows.
-  __device__ __forceinline__ void read(const SynthArgs& a, float2 (&v)[32], const int cfg, const int p) const {
+  // configuration slot cfg (annuli and labels: into acc, laid out as SynthArgs::acc). Every thread of
+  // the warp has read what it needs of the warp's X1 rows.
+  __device__ __forceinline__ void read(const SynthArgs& a, double* const acc, float2 (&v)[32], const int cfg, const int p) const {
     const int T = threadIdx.x;
     // forward 2D DFT of Psi_p (passes A, B, C)
     passA_fwd(v, tA);
@@ -2532,7 +2533,7 @@ struct Detect {
       if (T < a.n_det) {
         double tot = 0.0;
         for (int w = 0; w < kThreads / 32; ++w) tot += static_cast<double>(red[w * kMaxDet + T]);
-        a.acc[(static_cast<size_t>(a.cfg_base + cfg) * a.n_det + T) * a.n_probes + p] = tot * (1.0 / (kW * kW));
+        acc[(static_cast<size_t>(a.cfg_base + cfg) * a.n_det + T) * a.n_probes + p] = tot * (1.0 / (kW * kW));
       }
     } else if constexpr (MODE == kReadLabels) {
       // 3D STEM (Sec. 3.1): |DFT|^2 into a W x W plane, then each label's pixels summed by
@@ -2560,7 +2561,7 @@ struct Detect {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
         if (lane == 0)
-          a.acc[(static_cast<size_t>(a.cfg_base + cfg) * a.n_det + l) * a.n_probes + p] =
+          acc[(static_cast<size_t>(a.cfg_base + cfg) * a.n_det + l) * a.n_probes + p] =
               static_cast<double>(sum) * (1.0 / (kW * kW));
       }
     } else {
@@ -2787,7 +2788,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_synth_detect(const SynthArgs a)
 #pragma unroll
     for (int n1 = 0; n1 < 32; ++n1) v[n1] = tb[(lane_id >> 2) * 132 + 4 * n1 + (lane_id & 3)];
     __syncwarp();      // every lane has read its row before X1 overwrites the warp's rows
-    det.read(a, v, cfg, p);
+    det.read(a, a.acc, v, cfg, p);
   }
 }
 
@@ -2942,7 +2943,174 @@ __global__ void __launch_bounds__(kThreads, 1) k_synth_split(const SynthArgs a) 
       __syncwarp();      // every lane has read its row before X1 overwrites the warp's rows
       Detect<MODE> det;
       det.places(a, sm);
-      det.read(a, v, cfg, p);
+      det.read(a, a.acc, v, cfg, p);
+    }
+    __syncwarp();
+    split::arrive();
+  }
+  split::wait();
+}
+
+// The synthesis of four probe variants at once (partial coherence: the variants share the exit
+// waves and differ in their coefficients): a cluster of four CTAs per probe, split over the rows as
+// in k_synth_split, with the sums of all four variants in each thread, so that an exit-wave
+// element is loaded once for the four; CTA v then transforms and reads out variant v. Same
+// products in the same order as one launch per variant.
+//
+// What bounds it: issue and latency per wave (about 140 instructions for 64 packed FMAs), not the L2
+// port any more. 16384 probes, L = 32: 11.8 ms for four variants, 14.4 ms as four launches.
+namespace var {
+constexpr int kVar = kSynthVariants;
+constexpr int kMaxL = 64;
+constexpr int kBatch = 2;                // waves whose loads are in flight together
+constexpr int kSmemBytes = kSynthSmemFloat2 * 8 + kMaxL * (16 * kVar + 16);
+}  // namespace var
+
+// Annular detectors, non-periodic placement, L <= var::kMaxL; WS as in k_synth_detect.
+template <bool HALF, int WS>
+__global__ void __launch_bounds__(kThreads, 1) k_synth_variants(const SynthArgs a) {
+  extern __shared__ __align__(16) float2 sm[];
+  constexpr int C = 4, R = 2, NB = var::kBatch, V = var::kVar;
+  using Raw = typename std::conditional<HALF, uint2, float4>::type;
+  float4* const coef = reinterpret_cast<float4*>(sm + kSynthSmemFloat2);   // [L][V], cfma2's form
+  int4* const ent = reinterpret_cast<int4*>(coef + var::kMaxL * V);        // translate, placement
+  Detect<kReadAnnuli>::tables(sm);   // published by the barriers of the first item
+  float2* const R0 = sm;
+  const int T = threadIdx.x, warp = T >> 5, lane = T & 31;
+  int rank;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
+  const int Wu = WS > 0 ? WS : a.W;
+  const int y0 = R * (C * warp + rank);         // the warp's rows
+  const int n_items = a.n_probes * a.n_cfg;
+  split::arrive();
+  for (int item = blockIdx.x / C; item < n_items; item += gridDim.x / C) {
+    const int cfg = item / a.n_probes;
+    const int p = probe_of(item - cfg * a.n_probes, a.npx, a.npy, a.strip);
+    const size_t t0 = static_cast<size_t>(p) * a.L;
+    const float2* const Uc = a.U ? a.U + cfg * a.u_slot : nullptr;
+    const __half2* const Uhc = a.Uh ? static_cast<const __half2*>(a.Uh) + cfg * a.u_slot : nullptr;
+    const float* const Usc = a.Uscale ? a.Uscale + static_cast<size_t>(cfg) * a.n_translates : nullptr;
+    // the previous item's reads of the tables ended before its cluster barriers
+    if (T < V * a.L) {
+      const size_t e = t0 + T / V;
+      float2 al = a.alpha[(T % V) * a.alpha_stride + e];
+      if constexpr (HALF) {
+        const float f = Usc[a.tidx[e]];
+        al.x *= f;
+        al.y *= f;
+      }
+      coef[T] = make_float4(al.x, al.x, -al.y, al.y);
+    }
+    if (T < a.L) {
+      const int2 sh = a.shift[t0 + T];
+      ent[T] = make_int4(a.tidx[t0 + T], sh.x, sh.y, 0);
+    }
+    __syncthreads();
+    float2 acc[V][R][4];
+#pragma unroll
+    for (int v = 0; v < V; ++v)
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int m = 0; m < 4; ++m) acc[v][r][m] = make_float2(0.f, 0.f);
+    // lane l holds columns 64 kk + 2 l + e of the rows, as in k_synth_detect
+#pragma unroll 1
+    for (int j0 = 0; j0 < a.L; j0 += NB) {
+      Raw buf[NB][R][2];
+#pragma unroll
+      for (int b = 0; b < NB; ++b) {
+        const bool on = j0 + b < a.L;
+        const int4 e = ent[min(j0 + b, a.L - 1)];
+        const int yw = y0 - e.z, xw = 2 * lane - e.y;
+        const long long base = static_cast<long long>(e.x) * (Wu * Wu) + yw * Wu + xw;
+        const bool pair = (e.y & 1) == 0;    // column pairs stay aligned and unbroken
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          const bool oky = on && static_cast<unsigned>(yw + r) < static_cast<unsigned>(Wu);
+#pragma unroll
+          for (int kk = 0; kk < 2; ++kk) {
+            // only elements inside the window are read; the others count as zero
+            const bool k0 = oky && static_cast<unsigned>(xw + 64 * kk) < static_cast<unsigned>(Wu);
+            const bool k1 = oky && static_cast<unsigned>(xw + 64 * kk + 1) < static_cast<unsigned>(Wu);
+            const long long o = base + (r * Wu + 64 * kk);
+            Raw v{};
+            if constexpr (HALF) {
+              if (pair) {
+                if (k0) v = *reinterpret_cast<const uint2*>(Uhc + o);
+              } else {
+                if (k0) v.x = *reinterpret_cast<const unsigned*>(Uhc + o);
+                if (k1) v.y = *reinterpret_cast<const unsigned*>(Uhc + o + 1);
+              }
+            } else {
+              if (pair) {
+                if (k0) v = *reinterpret_cast<const float4*>(Uc + o);
+              } else {
+                if (k0) {
+                  const float2 f = Uc[o];
+                  v.x = f.x;
+                  v.y = f.y;
+                }
+                if (k1) {
+                  const float2 f = Uc[o + 1];
+                  v.z = f.x;
+                  v.w = f.y;
+                }
+              }
+            }
+            buf[b][r][kk] = v;
+          }
+        }
+      }
+#pragma unroll
+      for (int b = 0; b < NB; ++b) {
+        if (j0 + b >= a.L) break;
+        float2 f[R][4];
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+          for (int kk = 0; kk < 2; ++kk) {
+            if constexpr (HALF) {
+              f[r][2 * kk] = __half22float2(*reinterpret_cast<const __half2*>(&buf[b][r][kk].x));
+              f[r][2 * kk + 1] = __half22float2(*reinterpret_cast<const __half2*>(&buf[b][r][kk].y));
+            } else {
+              f[r][2 * kk] = make_float2(buf[b][r][kk].x, buf[b][r][kk].y);
+              f[r][2 * kk + 1] = make_float2(buf[b][r][kk].z, buf[b][r][kk].w);
+            }
+          }
+#pragma unroll
+        for (int v = 0; v < V; ++v) {
+          const float4 al4 = coef[(j0 + b) * V + v];
+#pragma unroll
+          for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int m = 0; m < 4; ++m) acc[v][r][m] = cfma2(acc[v][r][m], al4, f[r][m]);
+        }
+      }
+    }
+    split::wait();                               // every CTA of the cluster is past its last transform
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      const uint32_t dst = split::remote(R0, v);
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int y = y0 + r;
+#pragma unroll
+        for (int kk = 0; kk < 2; ++kk)
+          split::store4(dst + 8u * static_cast<uint32_t>((y >> 3) * (32 * 34) + (y & 7) * 132 + 64 * kk + 2 * lane), acc[v][r][2 * kk],
+                        acc[v][r][2 * kk + 1]);
+      }
+    }
+    split::arrive();
+    split::wait();
+    {
+      const float2* const tb = R0 + warp * (32 * 34);
+      float2 v[32];
+#pragma unroll
+      for (int n1 = 0; n1 < 32; ++n1) v[n1] = tb[(lane >> 2) * 132 + 4 * n1 + (lane & 3)];
+      __syncwarp();      // every lane has read its row before X1 overwrites the warp's rows
+      Detect<kReadAnnuli> det;
+      det.places(a, sm);
+      det.read(a, a.acc + rank * a.acc_stride, v, cfg, p);
     }
     __syncwarp();
     split::arrive();
@@ -3490,6 +3658,8 @@ cudaError_t init_device_constants() {
     for (int v = 0; v < 3; ++v)
       for (SynthKernel f : {synth_split_kernel<2>(v == 1, m, v == 2), synth_split_kernel<4>(v == 1, m, v == 2)})
         if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, sy)) != cudaSuccess) return e;
+  for (auto f : {k_synth_variants<false, 0>, k_synth_variants<false, kW>, k_synth_variants<true, kW>})
+    if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, var::kSmemBytes)) != cudaSuccess) return e;
   for (auto f : {k_synth_group<false>, k_synth_group<true>})
     if ((e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   static_cast<int>(synth_group_smem_bytes()))) != cudaSuccess)
@@ -3652,6 +3822,21 @@ static int split_clusters() {
     return cudaOccupancyMaxActiveClusters(&k, k_synth_split<false, kReadAnnuli, kW, C>, &cfg) == cudaSuccess ? k : 0;
   }();
   return n;
+}
+
+bool synth_variants_fit(const SynthArgs& a, bool half) {
+  return !a.cyclic && !a.probe_list && a.L <= var::kMaxL && a.W >= 32 && a.W <= 256 && (a.W == kW || !half) && split_clusters<4>() > 0;
+}
+cudaError_t launch_synth_variants(const SynthArgs& a, bool half, cudaStream_t s) {
+  if (!synth_variants_fit(a, half)) return cudaErrorInvalidValue;
+  const int n_items = a.n_probes * a.n_cfg;
+  if (n_items <= 0) return cudaSuccess;
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at{};
+  cluster_config(cfg, at, 4, n_items < split_clusters<4>() ? n_items : split_clusters<4>(), s);
+  cfg.dynamicSmemBytes = var::kSmemBytes;
+  const SynthKernel f = a.W != kW ? k_synth_variants<false, 0> : (half ? k_synth_variants<true, kW> : k_synth_variants<false, kW>);
+  return cudaLaunchKernelEx(&cfg, f, a);
 }
 
 cudaError_t launch_synth(const SynthArgs& a, bool half, int mode, int grid_mode, cudaStream_t s) {
