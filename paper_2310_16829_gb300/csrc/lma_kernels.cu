@@ -2,12 +2,15 @@
 //
 //   k_potential      step a1: v_s(x) = sum of Gaussian-sum atom potentials, t_s = exp(i sigma v_s)
 //                    (Sec. 3.2, transmission function)
-//   k_slice          step a3: multislice of each lattice translate u_i on its W x W window,
+//   k_slice          step a3: multislice of each lattice translate u_i on its W x W window (W = 128;
+//                    k_slice_64*, k_slice_256* the other windows, k_slice_tc on tensor cores),
 //                    transmit -> 2D FFT -> propagator and bandlimit -> inverse 2D FFT per slice
 //                    (Fig. multislice_pseudocode on the window of option (ii), Sec. 4.2.1)
 //   k_synth_detect   steps a4-a6: Psi_p = sum_j alpha_j U_{i_j} on the D x D probe window
 //                    (Sec. 4.2.2), |DFT(Psi_p)|^2 summed over the annular detector (Sec. 3.1),
 //                    FP64 accumulation over frozen-phonon configurations
+//                    (k_synth_split: small launches, a probe over a cluster of CTAs;
+//                    k_synth_variants: four probe variants over the same waves)
 //   k_finalize       step a6: average over configurations
 //
 // The 128 x 128 complex64 wave of one translate stays in registers of one
@@ -476,7 +479,7 @@ __device__ __forceinline__ void load_twiddles(float2* twA, float2* twB, int T) {
 // B and A, the transmission and forward A and B at its own pace, so that the exchanges of some
 // warps overlap the arithmetic of others. With warps of 8 consecutive window rows, X1 and X4
 // crossed warps (four barriers a slice) and the phases of all 16 warps ran in step: 320 ms
-// per 131072 translates x 50 slices, 291 ms since.
+// per 131072 translates x 50 slices, 291 ms since (289 with the twiddles in registers).
 // With rows of 34 entries the A side moves entry pairs (k, k + 1) with 128-bit accesses, a
 // quarter-warp's 8 rows on 8 distinct 16-byte slots (17 TA + k/2 mod 8); the 64-bit B and C
 // accesses of a half-warp are 16 consecutive entries of one row, on 16 distinct bank pairs (of
