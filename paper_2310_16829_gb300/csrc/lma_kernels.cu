@@ -378,6 +378,19 @@ __device__ __forceinline__ float2 tw_conj(float2 a, float s, float t) {
 // 44): forward it is not formed, inverse it is zero (C writes zeros there).
 template <bool COT, bool PRUNE>
 __host__ __device__ constexpr int masked_k2x() { return PRUNE ? (COT ? 1 : 2) : -1; }
+// Whether inverse pass B reads column kx. Pass C has to write every such column, also in the warps
+// that skip the propagation because all their columns lie outside the band: one warp of a k1y
+// group at radii 32..43, more below. (As a range of kx: 36.2 ms for 16384 translates x 50 slices; as
+// a condition on k1x and k2x 36.8, with unconditional writes 36.5.)
+template <bool PRUNE>
+__host__ __device__ constexpr bool passB_reads(int kx) { return !PRUNE || kx < 48 || kx >= 80; }
+constexpr bool passB_reads_fits_masked_k2x() {
+  for (int kx = 0; kx < 128; ++kx)
+    if (passB_reads<true>(kx) != ((kx >> 5) != ((kx & 31) < 16 ? masked_k2x<false, true>() : masked_k2x<true, true>())))
+      return false;
+  return true;
+}
+static_assert(passB_reads_fits_masked_k2x(), "pass C writes the columns that pass B reads");
 template <bool COT, bool PRUNE>
 __device__ __forceinline__ void passB_fwd_tw(float2 (&a)[16], const float2* twB, const float4 kA, const float4 kB) {
   constexpr int MC = masked_k2x<COT, PRUNE>();
@@ -655,8 +668,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_slice(const SliceLaunch a, cons
         dft32<true, PRUNE ? 2 : 0>(c);
 #pragma unroll
         for (int j = 0; j < 32; ++j) xc[j * 16 * kXP] = c[j];
-      } else if (!PRUNE || (k2x == 1 && k1x < 16)) {
-        // with PRUNE, pass B reads no other masked column of these warps (masked_k2x)
+      } else if (passB_reads<PRUNE>(kx)) {
 #pragma unroll
         for (int j = 0; j < 32; ++j) xc[j * 16 * kXP] = make_float2(0.f, 0.f);
       }
