@@ -1156,7 +1156,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_slice_tc(const SliceLaunch a, i
 #pragma unroll
           for (int k = 0; k < 16; ++k) xc[(16 * h + k) * 16 * kXP] = y[k];
         }
-      } else if (!PRUNE || (k2x == 1 && k1x < 16)) {   // the masked columns that pass B reads
+      } else if (passB_reads<PRUNE>(kx)) {
 #pragma unroll
         for (int j = 0; j < 32; ++j) xc[j * 16 * kXP] = make_float2(0.f, 0.f);
       }

@@ -72,3 +72,9 @@ def test_narrow_bandlimits_match_oracle(frac, offset, precision):
 @pytest.mark.parametrize("window", [64, 256])
 def test_narrow_bandlimits_of_other_windows_match_oracle(window, frac):
     _check(frac, window, WL.PREC_C64, 1 if frac == 0.3 else 2)
+
+
+@pytest.mark.parametrize("frac", FRACS)
+@pytest.mark.parametrize("offset", [1, 2])
+def test_narrow_bandlimits_on_tensor_cores_match_oracle(frac, offset):
+    _check(frac, 128, WL.PREC_MIXED, offset)
