@@ -3221,8 +3221,8 @@ lma_status lma_edit_column(lma_ctx* ctx, lma_specimen* sp, lma_basis* b, double 
         const int wy0 = mod(b->oy + ib * b->Sy - b->W / 2, g.ny);
         if (!meets(wy0, b->W, r.y0, r.h, g.ny)) continue;
         for (int ia = 0; ia < b->nax; ++ia) {
-          const int wx0 = mod(b->ox + ia * b->Sx - kW / 2, g.nx);
-          if (!meets(wx0, kW, r.x0, r.w, g.nx)) continue;
+          const int wx0 = mod(b->ox + ia * b->Sx - b->W / 2, g.nx);
+          if (!meets(wx0, b->W, r.x0, r.w, g.nx)) continue;
           const int64_t i = static_cast<int64_t>(ib) * b->nax + ia;
           for (int k = 0; k < b->B; ++k) {
             uint8_t& v = b->valid[static_cast<size_t>(k) * b->nT + i];
