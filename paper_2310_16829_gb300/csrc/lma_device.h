@@ -107,11 +107,11 @@ struct SynthArgs {
   // launch_synth_variants: variant v (of kSynthVariants) has its coefficients at alpha + v
   // alpha_stride and its readings at acc + v acc_stride
   size_t alpha_stride, acc_stride;
-  // kReadLabels: pixel lists of the labels (3D STEM rings), CSR over pixel ky * W + kx
+  // kReadLabels: pixel lists of the labels (3D STEM rings), CSR over pixel ky * D + kx
   const int32_t* lab_start;    // [n_det + 1]
   const int32_t* lab_pix;      // ascending pixel indices of each label
-  // kReadPattern: |DFT|^2 / W^2 at |kx| <= pat_a, |ky| <= pat_b (4D STEM), zero outside
-  // the band kx^2 + ky^2 <= band_r2, FP32 per configuration slot
+  // kReadPattern: |DFT|^2 / D^2 at |kx| <= pat_a, |ky| <= pat_b (4D STEM), zero outside
+  // the band kx^2 + ky^2 <= band_r2 of the D-grid, FP32 per configuration slot
   float* pat;                  // [slot][n_probes][2 pat_b + 1][2 pat_a + 1]
   int pat_a, pat_b;
   int band_r2;

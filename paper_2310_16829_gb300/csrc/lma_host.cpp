@@ -404,7 +404,8 @@ struct lma_basis {
   std::vector<cd> psi0;        // full-grid probe centred at pixel 0 (lazy)
   std::vector<cd> uW;          // W x W input wave
   std::vector<float> ex, ey;   // interleaved complex
-  int r2max = 0;
+  int r2max = 0;                 // bandlimit radius squared on the W-grid
+  int r2det = 0;                 // and on the D-grid of the readouts
   std::map<std::pair<int, int>, CoefSet> sets;
   // device
   DevBuf d_uW, d_ex, d_ey, d_U, d_Uscale, d_acc, d_det;
@@ -1710,7 +1711,7 @@ lma_status images_work(lma_ctx* ctx, const std::vector<ImageJob>& jobs, const Re
       a.det_bits = static_cast<const uint32_t*>(b->d_det.p);
       a.n_det = ro.n_out;
       a.acc = static_cast<double*>(b->d_acc.p);
-      a.band_r2 = b->r2max;
+      a.band_r2 = b->r2det;
       if (ro.mode == lma_dev::kReadLabels) {
         a.lab_start = static_cast<const int32_t*>(b->d_lab.p);
         a.lab_pix = a.lab_start + ro.n_out + 1;
@@ -2030,6 +2031,7 @@ lma_status lma_create_basis(lma_ctx* ctx, const lma_specimen* spec, const lma_pr
     b->ey[2 * m + 1] = static_cast<float>(std::sin(py));
   }
   b->r2max = bandlimit_r2(g.bandlimit_frac, b->W);
+  b->r2det = bandlimit_r2(g.bandlimit_frac, d.det_window);
   *out = b;
   return LMA_OK;
 }
@@ -2781,7 +2783,7 @@ lma_status lma_image_coherent(lma_ctx* ctx, lma_specimen* sp, lma_basis* b, cons
       a.det_bits = static_cast<const uint32_t*>(b->d_det.p);
       a.n_det = n_det;
       a.acc = static_cast<double*>(b->d_acc.p) + static_cast<size_t>(v) * nph * nout;
-      a.band_r2 = b->r2max;
+      a.band_r2 = b->r2det;
       // four variants in one launch where the gather serves them (no autotuning, no forced grouped form)
       if (n_var - v >= lma_dev::kSynthVariants && !ctx->autotune && ctx->synth_mode != LMA_SYNTH_GROUPED &&
           lma_dev::synth_variants_fit(a, half)) {
@@ -2906,7 +2908,7 @@ lma_status lma_image_partitioned(lma_ctx* ctx, lma_specimen* sp, lma_basis* b, c
       a.det_bits = static_cast<const uint32_t*>(b->d_det.p);
       a.n_det = n_det;
       a.acc = static_cast<double*>(b->d_acc.p);
-      a.band_r2 = b->r2max;
+      a.band_r2 = b->r2det;
       { const lma_status ss_ = synth_launch(ctx, a, half, lma_dev::kReadAnnuli, static_cast<int64_t>(P.probes.size()), SynthGeom{}, st); if (ss_ != LMA_OK) return ss_; }
     }
   }
