@@ -3839,8 +3839,13 @@ static int split_clusters() {
   return n;
 }
 
+// From four waves a probe on, or while one launch per variant would leave SMs idle. With fewer waves
+// the read-out outweighs the gather, and a cluster per probe keeps fewer probes in flight: 4096
+// probes, L = 1, 2, 3, 32 at W = 64 take 1194, 1212, 1295, 3214 us for four variants at once and 880,
+// 1018, 1191, 6048 us as four launches; 152 probes, L = 1: 58 us and 60.
 bool synth_variants_fit(const SynthArgs& a, bool half) {
-  return !a.cyclic && !a.probe_list && a.L <= var::kMaxL && a.W >= 32 && a.W <= 256 && (a.W == kW || !half) && split_clusters<4>() > 0;
+  return !a.cyclic && !a.probe_list && a.L <= var::kMaxL && a.W >= 32 && a.W <= 256 && (a.W == kW || !half) && split_clusters<4>() > 0 &&
+         (a.L >= 4 || a.n_probes * a.n_cfg <= sm_count());
 }
 cudaError_t launch_synth_variants(const SynthArgs& a, bool half, cudaStream_t s) {
   if (!synth_variants_fit(a, half)) return cudaErrorInvalidValue;

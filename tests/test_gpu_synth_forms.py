@@ -1,0 +1,48 @@
+"""The choice between the synthesis forms, by device time (CUDA events around the launches, the least
+of several averages): a call in the form that the library chooses, tuned or not, takes no longer than
+another form that it has for the same readings. The forms differ here by 1.3x or more where the
+choice matters; the tests allow 1.15x.
+"""
+import ctypes as C
+import dataclasses
+
+import numpy as np
+import pytest
+
+from paper_2310_16829_gb300 import lma, workloads as WL
+
+pytestmark = pytest.mark.gpu
+
+DETECTORS = [WL.Detector(0.0, 0.02), WL.Detector(0.03, 0.06)]
+
+
+def _basis(window, L):
+    w = WL.perovskite_workload(cells=5, nx=256, n_slices=1, n_phonons=1, seed_base=720)
+    ctx = lma.Context(0)
+    spec = lma.Specimen(ctx, w.grid, w.potential, w.phonons)
+    basis = lma.Basis(ctx, spec, w.probe, dataclasses.replace(w.basis, window=window, L=L))
+    basis.propagate(0)
+    return ctx, basis
+
+
+def _synth_ms(ctx, call, n=10):
+    for _ in range(3):
+        call()
+    best = np.inf
+    for _ in range(5):
+        ctx.profile_enable(True)
+        for _ in range(n):
+            call()
+        best = min(best, ctx.profile_read()["synth"]["total_ms"] / n)
+    ctx.profile_enable(False)
+    return best
+
+
+@pytest.mark.parametrize("window,L", [(64, 1), (64, 3), (128, 1), (64, 12)])
+def test_four_variants_take_no_longer_than_four_images(window, L):
+    ctx, basis = _basis(window, L)
+    region = WL.Region(7, 50, 64, 64, (4, 4))
+    series = [(10.0 * k, 0.0, 1.0) for k in range(4)]
+    four = _synth_ms(ctx, lambda: basis.image_coherent(series, DETECTORS, region))
+    one = _synth_ms(ctx, lambda: basis.image(DETECTORS, region))
+    assert four <= 1.15 * 4 * one, (window, L, four, one)
