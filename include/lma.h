@@ -534,7 +534,8 @@ lma_status lma_tuning_read(lma_ctx* ctx, lma_tuning* out, int32_t cap, int32_t* 
  * launch each, or for the grouped form the group and detection launches of every
  * configuration). Variants 0..5 are the per-probe gather, v = 2 s + g: strip width 16, 32, 64
  * for s = 0, 1, 2 (probes are walked in vertical strips of that many columns, which sets how
- * many exit waves the CTAs in flight share in L2) and grid g = 0 one CTA per probe, g = 1
+ * many exit waves the CTAs in flight share in L2) and grid g = 0 one CTA per probe (in launches
+ * of at most about half as many probes as SMs two, and of a quarter four CTAs, a cluster), g = 1
  * persistent (one CTA per SM walking the probes in order). Variants 6 and 7 are the grouped
  * form (LMA_SYNTH_GROUPED) with the group shapes group_shape[0] and group_shape[1] (ms 0 where
  * the launch does not admit it). Every variant gives the same readings bit for bit, so the
@@ -547,7 +548,7 @@ typedef struct {
   int32_t L;                 /* input waves per probe */
   int32_t window;            /* exit-wave window W */
   int32_t strip;             /* chosen strip width (gather) */
-  int32_t persistent;        /* chosen grid (gather): 1 persistent, 0 one CTA per probe */
+  int32_t persistent;        /* chosen grid (gather): 1 persistent, 0 one CTA (or cluster) per probe */
   int32_t grouped;           /* 1: the grouped form was chosen, with group_x x group_y probes */
   int32_t group_x, group_y;
   int32_t group_shape[2][2]; /* the two timed group shapes (x, y) of variants 6 and 7 */
@@ -558,7 +559,9 @@ typedef struct {
  * Both forms sum each probe's terms in ascending translate index and give the same readings
  * bit for bit. */
 #define LMA_SYNTH_AUTO -1     /* the tuned form of the launch shape, else the gather */
-#define LMA_SYNTH_GATHER 0    /* one CTA per probe gathers its L windows and detects */
+#define LMA_SYNTH_GATHER 0    /* one CTA per probe (small launches: a cluster of CTAs) gathers its L
+                                 windows and detects; lma_image_coherent may take four variants
+                                 of a probe in one launch */
 #define LMA_SYNTH_GROUPED 1   /* one CTA per group of up to 4 neighbouring probes loads each
                                  exit-wave element once for all of them and writes their waves
                                  to a device buffer (probes x 128 KiB, allocated by the

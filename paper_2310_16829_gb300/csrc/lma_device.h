@@ -152,8 +152,9 @@ size_t slice_gen_scratch_bytes(int W);
 // one warp runs the bounded mbarrier wait of the tensor-core (which = 0) or W = 256 (which = 1)
 // slice kernel on a phase that never completes; *status |= 1 when it gives up
 cudaError_t launch_selftest_wait(int which, int* status, cudaStream_t s);
-// synthesis grid: kSynthGridAuto (persistent for the complex64 store, one CTA per item for the
-// FP16 store), one CTA per item, or persistent (one CTA per SM); every grid gives the same bits
+// synthesis grid: persistent (one CTA per SM), one CTA per item (a cluster of two or four CTAs per item
+// where the launch would leave SMs idle), or kSynthGridAuto: per item for the FP16 store and for
+// such small launches, else persistent; every grid gives the same bits
 constexpr int kSynthGridAuto = 0, kSynthGridPerItem = 1, kSynthGridPersistent = 2;
 cudaError_t launch_synth(const SynthArgs& a, bool half, int mode, int grid_mode, cudaStream_t s);
 // annular readings of kSynthVariants coefficient sets over the same waves in one launch (the bits of

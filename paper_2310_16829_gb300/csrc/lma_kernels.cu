@@ -3874,7 +3874,7 @@ cudaError_t launch_synth(const SynthArgs& a, bool half, int mode, int grid_mode,
   // clusters of four lose to one CTA per probe (72 probes: 47 us against 38), so pairs take over,
   // and from half the SMs on k_synth_detect (81 probes: 38 us). A single wave per probe leaves nothing
   // to split (36 probes, W = 64: 16.2 us in clusters, 14.8 without; L = 3: 16.3 and 19.1).
-  if (grid_mode == kSynthGridAuto && !a.cyclic && a.L > 1 && n_items <= split_clusters<2>()) {
+  if (grid_mode != kSynthGridPersistent && !a.cyclic && a.L > 1 && n_items <= split_clusters<2>()) {
     if ((mode != kReadAnnuli && mode != kReadLabels && mode != kReadPattern) || (a.W != kW && (half || a.W < 32 || a.W > 256)))
       return cudaErrorInvalidValue;
     const bool four = n_items <= split_clusters<4>();

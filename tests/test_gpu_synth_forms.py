@@ -46,3 +46,16 @@ def test_four_variants_take_no_longer_than_four_images(window, L):
     four = _synth_ms(ctx, lambda: basis.image_coherent(series, DETECTORS, region))
     one = _synth_ms(ctx, lambda: basis.image(DETECTORS, region))
     assert four <= 1.15 * 4 * one, (window, L, four, one)
+
+
+def test_a_tuned_small_readout_takes_no_longer_than_an_untuned_one():
+    """36 probes with odd placements: a probe over a cluster of CTAs, tuned or not."""
+    ctx, basis = _basis(128, 32)
+    region = WL.Region(7, 50, 6, 6, (5, 5))
+    before = basis.image(DETECTORS, region)
+    untuned = _synth_ms(ctx, lambda: basis.image(DETECTORS, region))
+    assert np.array_equal(basis.image(DETECTORS, region, autotune=True), before)
+    assert len(ctx.synth_tuning()) == 1
+    tuned = _synth_ms(ctx, lambda: basis.image(DETECTORS, region))
+    assert np.array_equal(basis.image(DETECTORS, region), before)
+    assert tuned <= 1.15 * untuned, (tuned, untuned)
