@@ -99,6 +99,11 @@ struct lma_ctx {
     lma_synth_tuning rec;
   };
   std::vector<SynthTune> synth_tune;
+  struct VariantsTune {
+    std::vector<int64_t> key;
+    bool together;
+  };
+  std::vector<VariantsTune> variants_tune;   // kSynthVariants variants in one launch, or one launch each
   // captured image sequences (lma_image_many with LMA_IMAGE_GRAPH)
   struct Graph {
     std::vector<uintptr_t> key;
@@ -1199,6 +1204,53 @@ lma_status synth_launch(lma_ctx* ctx, lma_dev::SynthArgs& a, bool half, int mode
     tn.rec.persistent = best % 2;
   }
   ctx->synth_tune.push_back(tn);
+  return LMA_OK;
+}
+
+// Issue kSynthVariants variants over the same waves (coefficients and readings at the strides of a):
+// in one launch, or in one launch each (in the tuned form of that shape) where autotuning found
+// that faster for the shape. With autotuning on and a shape not seen before both run (each
+// assigns the same readings) and are timed with events on the stream.
+lma_status synth_variants(lma_ctx* ctx, const lma_dev::SynthArgs& a, bool half, int64_t units, const SynthGeom& geo,
+                          cudaStream_t st) {
+  auto together = [&]() -> lma_status {
+    CUDA_TRY(ctx, counted(ctx, K_SYNTH, units * lma_dev::kSynthVariants, st,
+                          [&] { return lma_dev::launch_synth_variants(a, half, st); }));
+    return LMA_OK;
+  };
+  auto apart = [&]() -> lma_status {
+    for (int v = 0; v < lma_dev::kSynthVariants; ++v) {
+      lma_dev::SynthArgs o = a;
+      o.alpha += v * a.alpha_stride;
+      o.acc += v * a.acc_stride;
+      const lma_status s = synth_launch(ctx, o, half, lma_dev::kReadAnnuli, units, geo, st);
+      if (s != LMA_OK) return s;
+    }
+    return LMA_OK;
+  };
+  const std::vector<int64_t> key{half ? 1 : 0, a.npx, a.npy, a.n_cfg, a.L, a.W, geo.psx, geo.psy};
+  const lma_ctx::VariantsTune* tuned = nullptr;
+  for (const auto& tt : ctx->variants_tune)
+    if (tt.key == key) tuned = &tt;
+  if (tuned || !ctx->autotune || ctx->capturing)
+    return tuned && !tuned->together && ctx->synth_mode == LMA_SYNTH_AUTO ? apart() : together();
+  lma_status s = apart();   // tunes the single launch where it has not been
+  if (s != LMA_OK) return s;
+  cudaEvent_t ev[3];
+  for (auto& e : ev) CUDA_TRY(ctx, cudaEventCreate(&e));
+  float ms[2] = {0.f, 0.f};
+  cudaError_t err = cudaEventRecord(ev[0], st);
+  if (err == cudaSuccess) s = apart();
+  if (err == cudaSuccess && s == LMA_OK) err = cudaEventRecord(ev[1], st);
+  if (err == cudaSuccess && s == LMA_OK) s = together();
+  if (err == cudaSuccess && s == LMA_OK) err = cudaEventRecord(ev[2], st);
+  if (err == cudaSuccess && s == LMA_OK) err = cudaEventSynchronize(ev[2]);
+  for (int i = 0; i < 2; ++i)
+    if (err == cudaSuccess && s == LMA_OK) err = cudaEventElapsedTime(&ms[i], ev[i], ev[i + 1]);
+  for (auto& e : ev) cudaEventDestroy(e);
+  if (s != LMA_OK) return s;
+  CUDA_TRY(ctx, err);
+  ctx->variants_tune.push_back({key, ms[1] <= ms[0]});
   return LMA_OK;
 }
 
@@ -2784,13 +2836,12 @@ lma_status lma_image_coherent(lma_ctx* ctx, lma_specimen* sp, lma_basis* b, cons
       a.n_det = n_det;
       a.acc = static_cast<double*>(b->d_acc.p) + static_cast<size_t>(v) * nph * nout;
       a.band_r2 = b->r2det;
-      // four variants in one launch where the gather serves them (no autotuning, no forced grouped form)
-      if (n_var - v >= lma_dev::kSynthVariants && !ctx->autotune && ctx->synth_mode != LMA_SYNTH_GROUPED &&
+      // four variants at once where the gather serves them (no forced grouped form)
+      if (n_var - v >= lma_dev::kSynthVariants && ctx->synth_mode != LMA_SYNTH_GROUPED &&
           lma_dev::synth_variants_fit(a, half)) {
         a.alpha_stride = static_cast<size_t>(np) * L;
         a.acc_stride = static_cast<size_t>(nph) * nout;
-        CUDA_TRY(ctx, counted(ctx, K_SYNTH, np * nb * lma_dev::kSynthVariants, st,
-                              [&] { return lma_dev::launch_synth_variants(a, half, st); }));
+        if ((s = synth_variants(ctx, a, half, np * nb, region_geom(b), st)) != LMA_OK) return s;
         v += lma_dev::kSynthVariants - 1;
         continue;
       }

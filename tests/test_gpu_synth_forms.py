@@ -59,3 +59,30 @@ def test_a_tuned_small_readout_takes_no_longer_than_an_untuned_one():
     tuned = _synth_ms(ctx, lambda: basis.image(DETECTORS, region))
     assert np.array_equal(basis.image(DETECTORS, region), before)
     assert tuned <= 1.15 * untuned, (tuned, untuned)
+
+
+def _coherent_autotuned(ctx, basis, series, region):
+    probes = (lma.Probe * len(series))(*[lma.Probe(basis.alpha_max, cs, dz) for dz, cs, _ in series])
+    weights = (C.c_double * len(series))(*[w for _, _, w in series])
+    dets = (lma.Detector * len(DETECTORS))(*[lma.Detector(d.r1, d.r2) for d in DETECTORS])
+    out = np.empty((len(DETECTORS), region.npy, region.npx), dtype=np.float64)
+    reg = lma.Region(region.px0, region.py0, region.npx, region.npy, (C.c_int32 * 2)(*region.spacing_px))
+    ctx.check(ctx.lib.lma_image_coherent(ctx.h, basis.spec.h, basis.h, probes, weights, len(series), dets,
+                                         len(DETECTORS), C.byref(reg), lma.LMA_IMAGE_AUTOTUNE,
+                                         out.ctypes.data_as(C.c_void_p), None))
+    return out
+
+
+@pytest.mark.parametrize("window,L", [(128, 32), (64, 48)])
+def test_a_tuned_focal_series_takes_no_longer_than_an_untuned_one(window, L):
+    """Nine variants (two launches of four and one of one) before, during and after tuning."""
+    ctx, basis = _basis(window, L)
+    region = WL.Region(7, 50, 12, 8, (4, 4))
+    series = [(10.0 * k, 0.0, 1.0 + k) for k in range(9)]
+    before = basis.image_coherent(series, DETECTORS, region)
+    untuned = _synth_ms(ctx, lambda: basis.image_coherent(series, DETECTORS, region))
+    assert np.array_equal(_coherent_autotuned(ctx, basis, series, region), before)
+    tuning = _synth_ms(ctx, lambda: _coherent_autotuned(ctx, basis, series, region))
+    tuned = _synth_ms(ctx, lambda: basis.image_coherent(series, DETECTORS, region))
+    assert np.array_equal(basis.image_coherent(series, DETECTORS, region), before)
+    assert tuned <= 1.15 * untuned and tuning <= 1.15 * untuned, (tuned, tuning, untuned)
