@@ -2094,7 +2094,9 @@ __global__ void __launch_bounds__(w64::kThreads64, 3) k_slice_64(const SliceLaun
 // g = warp / 2 the residue (pass 1) or k1 (pass 2); its passes work in place between CTA
 // barriers, and it writes its result transposed into the other buffer, so that the row phase runs
 // the column phase's code on B. The next slice's transmission is staged into a third buffer by
-// 8-byte cp.async while the column phase runs.
+// 8-byte cp.async while the column phase runs. Every product has the roundings stated in
+// k_slice_64: which kernel a list takes depends on its length, and short lists (edits, partitions)
+// stand beside long ones in one store.
 namespace w64w {
 using w64::c_tw;
 using w64::dft8;
@@ -2106,7 +2108,7 @@ constexpr int kBufE = kN * kP;           // float2 per buffer
 __device__ __forceinline__ void forward(float2* X, float2 (&v)[8], int c, int g) {
   dft8<false>(v);
 #pragma unroll
-  for (int k1 = 1; k1 < 8; ++k1) v[k1] = cmul(v[k1], c_tw[g * k1]);
+  for (int k1 = 1; k1 < 8; ++k1) v[k1] = cmul_yx(v[k1], c_tw[g * k1]);
 #pragma unroll
   for (int k1 = 0; k1 < 8; ++k1) X[(8 * k1 + g) * kP + c] = v[k1];
   __syncthreads();
@@ -2119,7 +2121,7 @@ __device__ __forceinline__ void forward(float2* X, float2 (&v)[8], int c, int g)
 __device__ __forceinline__ void inverse(float2* X, float2 (&v)[8], int c, int g) {
   dft8<true>(v);
 #pragma unroll
-  for (int q = 1; q < 8; ++q) v[q] = cmulc(v[q], c_tw[g * q]);
+  for (int q = 1; q < 8; ++q) v[q] = cmulc_y(v[q], c_tw[g * q]);
 #pragma unroll
   for (int q = 0; q < 8; ++q) X[(8 * g + q) * kP + c] = v[q];
   __syncthreads();
