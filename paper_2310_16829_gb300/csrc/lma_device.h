@@ -145,12 +145,11 @@ cudaError_t launch_slice_tc(const SliceLaunch& a, bool even_origins, cudaStream_
 size_t slice_tc_smem_bytes();
 // step a3 on W = 64 or W = 256 windows (every job of the launch has that W), complex64 store:
 // persistent CTAs (up to three per SM at W = 64, one at W = 256); even_origins as for
-// launch_slice (W = 64 uses it); W = 256 needs
-// slice_gen_scratch_bytes(256) of scratch
+// launch_slice; W = 256 needs slice_gen_scratch_bytes(256) of scratch
 cudaError_t launch_slice_gen(const SliceLaunch& a, bool even_origins, int W, float2* scratch, cudaStream_t s);
 size_t slice_gen_scratch_bytes(int W);
-// one warp runs the bounded mbarrier wait of the tensor-core (which = 0) or W = 256 (which = 1)
-// slice kernel on a phase that never completes; *status |= 1 when it gives up
+// one warp runs the bounded mbarrier wait of the tensor-core slice kernel (which = 0), or 16 warps that
+// of the W = 256 kernel for wide bandlimits (which = 1), on a phase that never completes; *status |= 1 when it gives up
 cudaError_t launch_selftest_wait(int which, int* status, cudaStream_t s);
 // synthesis grid: persistent (one CTA per SM), one CTA per item (a cluster of two or four CTAs per item
 // where the launch would leave SMs idle), or kSynthGridAuto: per item for the FP16 store and for

@@ -375,7 +375,7 @@ __device__ __forceinline__ float2 tw_conj(float2 a, float s, float t) {
 }
 // With PRUNE, column k2x = MC of this half lies outside the bandlimit for every ky
 // (k1 < 16: kx = k1 + 64, |kx| >= 49; k1 >= 16: kx = k1 + 32 >= 48; the radius is below
-// 44): forward it is not formed, inverse it is zero (C writes zeros there).
+// 44): forward it is not formed, inverse it is taken as zero.
 template <bool COT, bool PRUNE>
 __host__ __device__ constexpr int masked_k2x() { return PRUNE ? (COT ? 1 : 2) : -1; }
 // Whether inverse pass B reads column kx. Pass C has to write every such column, also in the warps
@@ -2817,7 +2817,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_synth_detect(const SynthArgs a)
 // same order. 2 (C = 2) or 5 (C = 4) waves' loads are in flight together, against one in
 // k_synth_detect, whose threads hold 32 sums instead of 16 or 8.
 //
-// What bounds it: latency, of the loads' L2 round trips and of the transform. One launch of L = 32,
+// What bounds it: latency, of the loads' L2 round trips and of the transform (issue 33 %, FMA pipe
+// 15 %, L2 22 %; barriers are the largest stall). One launch of L = 32,
 // complex64, 36 probes with even (odd) placements: 26 us (29), against 37 (87 with k_synth_detect's
 // odd placements one by one); 72 probes in clusters of two: 33 us (38), against 38 (88).
 namespace split {
@@ -2974,8 +2975,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_synth_split(const SynthArgs a) 
 // element is loaded once for the four; CTA v then transforms and reads out variant v. Same
 // products in the same order as one launch per variant.
 //
-// What bounds it: issue and latency per wave (about 140 instructions for 64 packed FMAs), not the L2
-// port any more. 16384 probes, L = 32: 11.8 ms for four variants, 14.4 ms as four launches.
+// What bounds it: issue and latency per wave (206 instructions of a warp, the transform's share
+// included, for 64 packed FMAs: issue 47 %, FMA pipe 42 %), not the L2 port any more (23 %). 16384
+// probes, L = 32: 11.8 ms for four variants, 14.4 ms as four launches.
 namespace var {
 constexpr int kVar = kSynthVariants;
 constexpr int kMaxL = 64;
@@ -3767,7 +3769,7 @@ cudaError_t launch_slice_gen(const SliceLaunch& a, bool even_origins, int W, flo
       (even_origins ? k_slice_64<true> : k_slice_64<false>)<<<units < 3 * sms ? units : 3 * sms, w64::kThreads64, w64::kSmemBytes, s>>>(a, units);
   } else if (W == 256) {
     if (!scratch) return cudaErrorInvalidValue;
-bool prune = true;   // k_slice_256 needs every job's bandlimit radius below 86 pixels
+    bool prune = true;   // k_slice_256 needs every job's bandlimit radius below 86 pixels
     for (int i = 0; i < a.n_jobs; ++i) prune = prune && a.job[i].r2max < 86 * 86;
     if (prune)
       (even_origins ? k_slice_256<true> : k_slice_256<false>)<<<grid, 512, w256p::kSmemBytes, s>>>(a, scratch);
